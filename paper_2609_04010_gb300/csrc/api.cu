@@ -212,7 +212,7 @@ spec_status_t check_lm_head(const spec_lm_head_args_t* a) {
     return SPEC_ERR_INVALID_ARGUMENT;
   if ((reinterpret_cast<uintptr_t>(a->hidden_states) | reinterpret_cast<uintptr_t>(a->weight)) & 15u)
     return SPEC_ERR_INVALID_ARGUMENT;
-  if ((a->vocab + kLmTileN - 1) / kLmTileN > 65535) return SPEC_ERR_UNSUPPORTED;  // grid y
+  if (a->vocab > kLmMaxVocab) return SPEC_ERR_UNSUPPORTED;
   return SPEC_OK;
 }
 
@@ -663,7 +663,7 @@ spec_status_t spec_lm_head_stats(const spec_lm_head_args_t* a, void* ws, size_t 
   cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_);
   DeviceScope scope(stream);
   if (!scope.ok) return SPEC_ERR_CUDA;
-  return launch_lm_head(*a, L, static_cast<char*>(ws), stream) == cudaSuccess ? SPEC_OK : SPEC_ERR_CUDA;
+  return launch_lm_head(*a, L, static_cast<char*>(ws), scope.sms, stream) == cudaSuccess ? SPEC_OK : SPEC_ERR_CUDA;
 }
 
 spec_status_t spec_test_lm_head_wait_timeout(const spec_lm_head_args_t* a, void* ws,
@@ -676,7 +676,7 @@ spec_status_t spec_test_lm_head_wait_timeout(const spec_lm_head_args_t* a, void*
   cudaStream_t stream = reinterpret_cast<cudaStream_t>(stream_);
   DeviceScope scope(stream);
   if (!scope.ok) return SPEC_ERR_CUDA;
-  return launch_lm_head(*a, L, static_cast<char*>(ws), stream, /*starve=*/true) == cudaSuccess
+  return launch_lm_head(*a, L, static_cast<char*>(ws), scope.sms, stream, /*starve=*/true) == cudaSuccess
              ? SPEC_OK
              : SPEC_ERR_CUDA;
 }

@@ -93,3 +93,58 @@ def test_lm_head_token_edges_and_bad_rows(oracle_mod):
     o = oracle_mod.lm_head_stats(h, w, T, 4, tokens=tok, rows=good)
     np.testing.assert_array_equal(g["row_argmax"][good], o["row_argmax"])
     assert abs(g["token_logit"][3] - o["token_logit"][good.index(3)]) < 1e-3
+
+
+# One block per row tile up to 128 rows, two above; vocabularies that leave a tile of one
+# 16-row unit, a ragged last unit, tiles of two sizes, and fewer tiles than SMs.
+@pytest.mark.parametrize("R,H,V,rps", [(128, 72, 16 * 152 + 1, 16), (129, 72, 31, 16), (256, 136, 40001, 16),
+                                       (257, 64, 8192, 1), (700, 200, 77777, 7), (5, 4096, 39000, 1)])
+def test_lm_head_tile_plan_edges(oracle_mod, R, H, V, rps):
+    h, w, T, tok = W.make_lm_inputs(R, H, V, rps, temperature=[1.0, 0.7], seed=R + V)
+    rows = sorted({0, 1, R // 2, min(R, 128) - 1, R - 1, min(R - 1, 255), min(R - 1, 256)})
+    check(oracle_mod, h, w, T, rps, tok, rows=rows)
+
+
+@pytest.mark.parametrize("R,V", [(260, 3000), (130, 2999)])
+def test_lm_head_pair_logits_output(oracle_mod, R, V):
+    h, w, T, tok = W.make_lm_inputs(R, 256, V, 8, seed=8)
+    g = gpu_lm(h, w, T, 8, tok, want_logits=True)
+    o = oracle_mod.lm_head_stats(h, w, T, 8, tokens=tok)
+    err = 2.0 ** -20 * o["abs_bound"][:, None]
+    assert np.all(np.abs(g["logits"] - o["logits"]) <= np.abs(o["logits"]) * 2.0 ** -8 + err + 1e-30)
+
+
+def test_lm_head_pair_bad_row_and_repeated_maximum():
+    # a NaN marks its own row only; equal maxima far apart keep the lowest index
+    R, H, V = 200, 64, 50000
+    h, w, T, tok = W.make_lm_inputs(R, H, V, 8, seed=9)
+    h, w = h.copy(), w.copy()
+    h[150, 3] = np.uint16(0x7FC0)
+    at = [17, 9000, 49999]
+    w[at] = h[20]  # the row itself: its largest logit, three times
+    ws = binding.new_workspace(1 << 24)
+    r = binding.lm_head_stats(bf16_dev(h), bf16_dev(w), dev(T), 8, tokens=dev(tok), ws=ws)
+    torch.cuda.synchronize()
+    assert binding.read_device_status(ws)[1] == binding.FLAG_BAD_LOGITS
+    arg = r["row_argmax"].cpu().numpy()
+    assert arg[150] == -1 and np.all(arg[np.arange(R) != 150] >= 0)
+    assert arg[20] == 17
+
+
+def test_lm_head_pair_wait_runs_out():
+    R, H, V = 300, 256, 9000
+    h, w, T, tok = W.make_lm_inputs(R, H, V, 8, seed=94)
+    out = dict(row_max=torch.empty(R, device="cuda"), row_sum=torch.empty(R, device="cuda"),
+               row_argmax=torch.empty(R, dtype=torch.int32, device="cuda"), token_logit=None)
+    keep = (bf16_dev(h), bf16_dev(w), dev(T))
+    a = binding.lm_head_args(*keep, 8, out)
+    ws = binding.new_workspace(binding.lm_head_workspace_size(a))
+    binding.test_lm_head_wait_timeout_args(a, ws)
+    torch.cuda.synchronize()
+    code, flags = binding.read_device_status(ws)
+    assert code == 6 and flags & binding.FLAG_TIMEOUT
+    binding.lm_head_stats_args(a, ws)
+    torch.cuda.synchronize()
+    assert binding.read_device_status(ws) == (0, 0)
+    ref = keep[0].double() @ keep[1].double().T
+    assert torch.equal(out["row_argmax"].long().cpu(), ref.argmax(-1).cpu())
