@@ -76,7 +76,10 @@ typedef enum { SPEC_F32 = 0, SPEC_BF16 = 1 } spec_dtype_t;
 
 /* Attention kernel selection (spec_attn_args_t.path). */
 typedef enum {
-  SPEC_ATTN_AUTO = 0,          /* tensor cores when (Hq/Hkv)*gamma >= the crossover, else CUDA cores */
+  SPEC_ATTN_AUTO = 0,          /* tensor cores when (Hq/Hkv)*gamma >= the crossover, else CUDA cores:
+                                  up to 32 query rows per KV head and an even Hkv, the
+                                  small-group kernel (several KV heads per block, register
+                                  accumulators); else as 2                               */
   SPEC_ATTN_CUDA_CORES = 1,    /* fp32 CUDA-core kernel                                  */
   SPEC_ATTN_TENSOR_CORES = 2,  /* tcgen05 (TMEM accumulators, TMA-staged KV pages), the
                                   row-tile kernel (M = 128 query rows per tile); with 33

@@ -245,8 +245,10 @@ spec_status_t check_accept(const spec_accept_args_t* a) {
 AttnPlan attn_plan(const spec_attn_args_t& a, size_t base, int num_sms, int path_override) {
   AttnPlan P;
   P.head_pair = 0;
+  P.heads = 0;
   P.rows = (a.num_q_heads / a.num_kv_heads) * a.gamma;
   int path = path_override;
+  if (path == SPEC_ATTN_AUTO && a.batch <= kTcMaxBatch) P.heads = mma_heads(a, P.rows);
   if (path == SPEC_ATTN_AUTO)
     path = (P.rows >= tc_min_rows() && a.batch <= kTcMaxBatch) ? SPEC_ATTN_TENSOR_CORES
                                                                : SPEC_ATTN_CUDA_CORES;
@@ -274,6 +276,17 @@ AttnPlan attn_plan(const spec_attn_args_t& a, size_t base, int num_sms, int path
     P.grid = 0;
     P.slot_rows = P.rows_per_cta;
     P.slots = P.nsplit > 1 ? units * P.nsplit : 0;
+  } else if (P.heads > 0) {
+    // persistent grid, one block per SM; one unit per (sequence, group of KV heads)
+    P.rows_per_cta = P.rows;
+    P.key_tile = 0;
+    P.row_tiles = 1;
+    units = static_cast<int64_t>(a.batch) * (a.num_kv_heads / P.heads);
+    P.nsplit = 1;
+    P.tiles_per_split = 0;
+    P.grid = num_sms;
+    P.slot_rows = P.heads * P.rows;
+    P.slots = units + P.grid;
   } else if (P.keys_on_lanes) {
     // persistent grid, one block per SM; one unit per (sequence, KV head)
     P.rows_per_cta = kKlMaxRows;
@@ -315,8 +328,9 @@ namespace {
 
 size_t attn_region(const spec_attn_args_t& a, size_t base, int sms) {
   size_t end = base;
-  for (int path : {SPEC_ATTN_CUDA_CORES, SPEC_ATTN_TENSOR_CORES, SPEC_ATTN_TENSOR_CORES_KEYS_ON_LANES}) {
-    if (path != SPEC_ATTN_CUDA_CORES && a.batch > kTcMaxBatch) continue;
+  for (int path : {SPEC_ATTN_AUTO, SPEC_ATTN_CUDA_CORES, SPEC_ATTN_TENSOR_CORES,
+                   SPEC_ATTN_TENSOR_CORES_KEYS_ON_LANES}) {
+    if (path != SPEC_ATTN_CUDA_CORES && path != SPEC_ATTN_AUTO && a.batch > kTcMaxBatch) continue;
     const AttnPlan P = attn_plan(a, base, sms, path);
     if (P.end > end) end = P.end;
   }
@@ -400,6 +414,7 @@ spec_status_t run(const spec_attn_args_t* attn, const spec_accept_args_t* accept
     if (!attn) return true;
     const AttnPlan P = attn_plan(*attn, attn_base, sms, attn->path);
     const cudaError_t e = P.path != SPEC_ATTN_TENSOR_CORES ? launch_attn_simt(*attn, P, w, stream)
+                          : P.heads > 0                     ? launch_attn_mma(*attn, P, w, stream)
                           : P.keys_on_lanes                 ? launch_attn_kl(*attn, P, w, stream)
                                                             : launch_attn_tc(*attn, P, w, stream);
     return e == cudaSuccess;

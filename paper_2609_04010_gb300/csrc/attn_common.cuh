@@ -15,8 +15,8 @@ namespace specv {
 
 struct AttnParams {
   int batch, gamma, hq, hkv, group, rows, row_tiles, rows_per_cta;
-  int hunits;        // KV-head units per sequence: Hkv, or Hkv / 2 when a block serves
-                     // two adjacent KV heads together (tensor-core head-pair variant)
+  int hunits;        // KV-head units per sequence: Hkv over the adjacent KV heads that one
+                     // block serves together
   int page_size, max_pages, num_pages;
   int nsplit, tiles_per_split;
   int slot_rows;     // rows stored per partial slot
@@ -36,6 +36,8 @@ struct AttnParams {
   int q_tma;           // tensor-core kernel: Q tiles arrive by TMA (else softmax warps load them)
   int unit_overhead;   // tensor-core kernel: tiles charged per unit start in the work list
   const uint64_t* tree_mask;  // [batch][gamma] block keys each query sees, or NULL (causal)
+  int grid, min_tiles; // range_count: blocks launched, tiles a block takes at least
+  int unit_heads;      // KV heads of a unit (attn_merge_kernel)
   int starve;  // test hook: the producers issue no copies, so the consumers' waits run out
 };
 
@@ -45,7 +47,7 @@ inline AttnParams make_attn_params(const spec_attn_args_t& a, const AttnPlan& P,
   p.gamma = a.gamma;
   p.hq = a.num_q_heads;
   p.hkv = a.num_kv_heads;
-  p.hunits = P.head_pair ? a.num_kv_heads / 2 : a.num_kv_heads;
+  p.hunits = P.heads > 0 ? a.num_kv_heads / P.heads : P.head_pair ? a.num_kv_heads / 2 : a.num_kv_heads;
   p.group = a.num_q_heads / a.num_kv_heads;
   p.rows = P.rows;
   p.row_tiles = P.row_tiles;
@@ -74,6 +76,9 @@ inline AttnParams make_attn_params(const spec_attn_args_t& a, const AttnPlan& P,
   p.unit_overhead = 0;
   p.tree_mask = a.tree_mask;
   p.starve = 0;
+  p.grid = P.grid;
+  p.min_tiles = 1;
+  p.unit_heads = 1;
   return p;
 }
 
@@ -263,6 +268,200 @@ __device__ void merge_unit(const AttnParams& p, int b, int g, int row0, int nrow
       if (c8 == 0) write_lse(p, b, g, row0 + r, M[i], L[i], dead);
     }
   }
+}
+
+// Contiguous global -> shared copy by the copy engine, completing on bar (16-byte aligned
+// addresses, size a multiple of 16).
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+// Orders this thread's view of global memory (generic proxy) before its later copies
+// by the copy engine (async proxy).
+__device__ __forceinline__ void fence_async_global() {
+  asm volatile("fence.proxy.async.global;" ::: "memory");
+}
+
+// Merge of one unit from its partial slots staged in shared memory: so[nsl][slot_rows][D]
+// and sml[nsl][slot_rows] = (m, l), row r of [row0, row0 + nrows) at slot row prow0 + r.
+// The same combination as merge_unit, with every load from shared memory.
+template <int D>
+__device__ void merge_staged(const AttnParams& p, int b, int g, int row0, int nrows, const float* so,
+                             const float2* sml, int nsl, int prow0, int tid, int nthreads) {
+  constexpr int C8 = D / 8;
+  for (int idx = tid; idx < nrows * C8; idx += nthreads) {
+    const int r = idx / C8, c8 = idx % C8, pr = prow0 + r;
+    float mx = -INFINITY;
+    bool bad = false;
+    for (int i = 0; i < nsl; ++i) {
+      const float2 ml = sml[i * p.slot_rows + pr];
+      bad |= ml.y < 0.f;
+      if (ml.y > 0.f) mx = fmaxf(mx, ml.x);
+    }
+    float L = 0.f, acc[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) acc[e] = 0.f;
+    if (mx != -INFINITY) {
+      for (int i = 0; i < nsl; ++i) {
+        const float2 ml = sml[i * p.slot_rows + pr];
+        if (!(ml.y > 0.f)) continue;
+        const float w = ex2(ml.x - mx);
+        const float4* src = reinterpret_cast<const float4*>(so + (static_cast<size_t>(i) * p.slot_rows + pr) * D) + 2 * c8;
+        const float4 a = src[0], c = src[1];
+        L += ml.y * w;
+        acc[0] += a.x * w; acc[1] += a.y * w; acc[2] += a.z * w; acc[3] += a.w * w;
+        acc[4] += c.x * w; acc[5] += c.y * w; acc[6] += c.z * w; acc[7] += c.w * w;
+      }
+    }
+    const bool dead = bad || !(L > 0.f);
+    write_out_row<D>(p, b, g, row0 + r, c8 * 8, acc, dead ? 0.f : 1.f / L);
+    if (c8 == 0) write_lse(p, b, g, row0 + r, mx, L, dead);
+  }
+}
+
+// ---------------------------------------------------------------------------------
+// Merging split units in a kernel of their own
+// ---------------------------------------------------------------------------------
+// pb[b] = virtual tiles of the sequences before b (one warp).
+template <int TK>
+__device__ __forceinline__ void tile_prefix(const AttnParams& p, int* pb, int lane) {
+  const int per_b = p.hunits * p.row_tiles;
+  int carry = 0;
+  for (int b0 = 0; b0 < p.batch; b0 += 32) {
+    const int b = b0 + lane;
+    int v = b < p.batch ? (unit_tiles<TK>(p.kv_len[b], p) + p.unit_overhead) * per_b : 0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, v, o);
+      if (lane >= o) v += y;
+    }
+    if (b < p.batch) pb[b + 1] = carry + v;
+    carry += __shfl_sync(0xffffffffu, v, 31);
+  }
+  if (lane == 0) pb[0] = 0;
+}
+
+// Ranges the virtual tiles are cut into: one per block, of at least min_tiles tiles each
+// (below that a block's start, partial and merge cost more than the tiles it takes off the
+// others).
+__device__ __forceinline__ int range_count(int64_t total, const AttnParams& p) {
+  const int64_t want = (total + p.min_tiles - 1) / p.min_tiles;
+  return want < p.grid ? static_cast<int>(want) : p.grid;
+}
+
+// The outputs of the units that were split between blocks, from their partial slots. Block
+// (c, y) stands for the boundary before range c + 1: the k-th boundary inside a unit merges
+// the k-th share of the unit's rows (of gridDim.y pieces, piece y), so that every block
+// reads about one slot however many ways a unit was split. One warp takes a row at a time;
+// its loads of all slots are in flight together. Merging in the last block of a unit to
+// finish instead (atomic ticket) left most SMs idle while a few read every slot: 3 us for
+// the fence and the ticket and 7 to 15 us for the merge (8 requests of 32 rows per KV head
+// and 4,096 keys: 53.3 us; here 37.2).
+constexpr int kAttnMergeThreads = 256;
+constexpr int kAttnMergePieces = 2;
+template <int D, int TK>
+__global__ void __launch_bounds__(kAttnMergeThreads) attn_merge_kernel(AttnParams p) {
+  extern __shared__ int pb_sh[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (warp == 0) tile_prefix<TK>(p, pb_sh, lane);
+  __syncthreads();
+  const int64_t total = pb_sh[p.batch];
+  const int ctas = range_count(total, p);
+  const int c = blockIdx.x + 1;
+  if (c >= ctas) return;
+  const Seg s = locate<TK>(static_cast<int64_t>(c) * total / ctas, total, p, pb_sh, p.unit_overhead);
+  // the boundary lies inside the unit's real tiles
+  if (static_cast<int64_t>(c) * total / ctas <= s.unit_start) return;
+  const int c_first = owner_of(s.unit_start, total, ctas);
+  const int nsl = owner_of(s.unit_start + s.unit_tiles - 1, total, ctas) - c_first + 1;
+  const int rows = min(p.slot_rows, p.unit_heads * min(p.rows_per_cta, p.rows - s.rt * p.rows_per_cta));
+  const int parts = (nsl - 1) * gridDim.y, part = (c - c_first - 1) * gridDim.y + blockIdx.y;
+  const int r_end = static_cast<int>(static_cast<int64_t>(rows) * (part + 1) / parts);
+  const int head_rows = rows / p.unit_heads;  // a unit's heads follow each other in a slot
+  const int64_t slot0 = s.u + c_first;
+  constexpr int E = D / 32;  // output columns per lane
+  constexpr int SB = 8;      // slots whose loads are in flight together
+  pdl_wait_prior();
+  for (int r = static_cast<int>(static_cast<int64_t>(rows) * part / parts) + warp; r < r_end;
+       r += kAttnMergeThreads / 32) {
+    float M = -INFINITY, L = 0.f, acc[E];
+    bool bad = false;
+#pragma unroll
+    for (int e = 0; e < E; ++e) acc[e] = 0.f;
+    for (int s0 = 0; s0 < nsl; s0 += SB) {
+      float2 ml[SB];
+      float o[SB][E];
+#pragma unroll
+      for (int i = 0; i < SB; ++i) {
+        const int64_t row = (slot0 + s0 + i) * p.slot_rows + r;
+        ml[i] = make_float2(-INFINITY, 0.f);
+#pragma unroll
+        for (int e = 0; e < E; ++e) o[i][e] = 0.f;
+        if (s0 + i < nsl) {
+          ml[i] = __ldcg(&p.partial_ml[row]);
+          if (E == 4) {
+            const float4 v = __ldcg(reinterpret_cast<const float4*>(p.partial_o + row * D) + lane);
+            o[i][0] = v.x; o[i][1] = v.y; o[i][E - 2] = v.z; o[i][E - 1] = v.w;
+          } else {
+            const float2 v = __ldcg(reinterpret_cast<const float2*>(p.partial_o + row * D) + lane);
+            o[i][0] = v.x; o[i][1] = v.y;
+          }
+        }
+      }
+      float mb = M;
+#pragma unroll
+      for (int i = 0; i < SB; ++i) {
+        bad |= ml[i].y < 0.f;
+        if (ml[i].y > 0.f) mb = fmaxf(mb, ml[i].x);
+      }
+      if (mb == -INFINITY) continue;
+      const float scale = M == -INFINITY ? 0.f : ex2(M - mb);
+      L *= scale;
+#pragma unroll
+      for (int e = 0; e < E; ++e) acc[e] *= scale;
+#pragma unroll
+      for (int i = 0; i < SB; ++i) {
+        if (!(ml[i].y > 0.f)) continue;
+        const float w = ex2(ml[i].x - mb);
+        L += ml[i].y * w;
+#pragma unroll
+        for (int e = 0; e < E; ++e) acc[e] += o[i][e] * w;
+      }
+      M = mb;
+    }
+    const bool dead = bad || !(L > 0.f);
+    const float inv = dead ? 0.f : 1.f / L;
+    const int kvh = s.g * p.unit_heads + r / head_rows, row = s.rt * p.rows_per_cta + r % head_rows;
+    const int j = row / p.group, h = kvh * p.group + row % p.group;
+    uint32_t w[E / 2];
+#pragma unroll
+    for (int e = 0; e < E / 2; ++e) {
+      const __nv_bfloat162 v = __floats2bfloat162_rn(dead ? 0.f : acc[2 * e] * inv, dead ? 0.f : acc[2 * e + 1] * inv);
+      w[e] = *reinterpret_cast<const uint32_t*>(&v);
+    }
+    __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(p.out) +
+                         ((static_cast<int64_t>(s.b) * p.gamma + j) * p.hq + h) * D + lane * E;
+    if (E == 4) *reinterpret_cast<uint2*>(dst) = make_uint2(w[0], w[E / 2 - 1]);
+    else *reinterpret_cast<uint32_t*>(dst) = w[0];
+    if (lane == 0) write_lse(p, s.b, kvh, row, M, L, dead);
+  }
+}
+
+template <int D, int TK>
+cudaError_t launch_merge(const AttnParams& p, cudaStream_t stream) {
+  if (p.grid < 2) return cudaSuccess;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(p.grid - 1, kAttnMergePieces);
+  cfg.blockDim = dim3(kAttnMergeThreads);
+  cfg.dynamicSmemBytes = 4u * (p.batch + 1);
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, attn_merge_kernel<D, TK>, p);
 }
 #endif
 

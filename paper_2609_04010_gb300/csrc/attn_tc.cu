@@ -151,58 +151,9 @@ __device__ __forceinline__ void tma_load_q(uint32_t dst, const CUtensorMap* map,
       "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(half), "r"(head0), "r"(pos0), "r"(bar)
       : "memory");
 }
-// Contiguous global -> shared copy by the copy engine, completing on bar (16-byte aligned
-// addresses, size a multiple of 16).
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-               "l"(src), "r"(bytes), "r"(bar)
-               : "memory");
-}
-// Orders this thread's view of global memory (generic proxy) before its later copies
-// by the copy engine (async proxy).
-__device__ __forceinline__ void fence_async_global() {
-  asm volatile("fence.proxy.async.global;" ::: "memory");
-}
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<const uint32_t*>(&v);
-}
-
-// Merge of one unit from its partial slots staged in shared memory: so[nsl][slot_rows][D]
-// and sml[nsl][slot_rows] = (m, l), row r of [row0, row0 + nrows) at slot row prow0 + r.
-// The same combination as merge_unit, with every load from shared memory.
-template <int D>
-__device__ void merge_staged(const AttnParams& p, int b, int g, int row0, int nrows, const float* so,
-                             const float2* sml, int nsl, int prow0, int tid, int nthreads) {
-  constexpr int C8 = D / 8;
-  for (int idx = tid; idx < nrows * C8; idx += nthreads) {
-    const int r = idx / C8, c8 = idx % C8, pr = prow0 + r;
-    float mx = -INFINITY;
-    bool bad = false;
-    for (int i = 0; i < nsl; ++i) {
-      const float2 ml = sml[i * p.slot_rows + pr];
-      bad |= ml.y < 0.f;
-      if (ml.y > 0.f) mx = fmaxf(mx, ml.x);
-    }
-    float L = 0.f, acc[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) acc[e] = 0.f;
-    if (mx != -INFINITY) {
-      for (int i = 0; i < nsl; ++i) {
-        const float2 ml = sml[i * p.slot_rows + pr];
-        if (!(ml.y > 0.f)) continue;
-        const float w = ex2(ml.x - mx);
-        const float4* src = reinterpret_cast<const float4*>(so + (static_cast<size_t>(i) * p.slot_rows + pr) * D) + 2 * c8;
-        const float4 a = src[0], c = src[1];
-        L += ml.y * w;
-        acc[0] += a.x * w; acc[1] += a.y * w; acc[2] += a.z * w; acc[3] += a.w * w;
-        acc[4] += c.x * w; acc[5] += c.y * w; acc[6] += c.z * w; acc[7] += c.w * w;
-      }
-    }
-    const bool dead = bad || !(L > 0.f);
-    write_out_row<D>(p, b, g, row0 + r, c8 * 8, acc, dead ? 0.f : 1.f / L);
-    if (c8 == 0) write_lse(p, b, g, row0 + r, mx, L, dead);
-  }
 }
 
 // ---------------------------------------------------------------------------------

@@ -138,6 +138,7 @@ cudaError_t launch_tree_build(const spec_tree_build_args_t& t, const TreeBuildLa
 struct AttnPlan {
   int path;          // SPEC_ATTN_CUDA_CORES or SPEC_ATTN_TENSOR_CORES
   int keys_on_lanes; // tensor cores: the keys-on-lanes kernel (attn_kl.cu), else row tiles
+  int heads;         // > 0: the small-group kernel (attn_mma.cu) with this many KV heads per block
   int head_pair;     // row tiles: one block serves two adjacent KV heads (8 KB page boxes)
   int rows;          // (Hq/Hkv) * gamma
   int rows_per_cta;  // rows one block handles (a row tile)
@@ -174,6 +175,14 @@ cudaError_t launch_attn_simt(const spec_attn_args_t& a, const AttnPlan& P, char*
 // run out and it returns with SPEC_FLAG_TIMEOUT set.
 cudaError_t launch_attn_tc(const spec_attn_args_t& a, const AttnPlan& P, char* ws,
                            cudaStream_t stream, bool starve = false);
+cudaError_t launch_attn_mma(const spec_attn_args_t& a, const AttnPlan& P, char* ws,
+                            cudaStream_t stream);
+// KV heads one block of the small-group kernel serves (2, 4 or 8), or 0 where it does not
+// apply: more than kMmaMaxRows query rows per KV head, an odd Hkv, or a batch whose prefix
+// sums do not fit beside its stages.
+int mma_heads(const spec_attn_args_t& a, int rows);
+constexpr int kMmaMaxRows = 32;
+constexpr int kMmaMinTiles = 2;  // 32 KB tiles a block takes at least (range_count)
 cudaError_t launch_attn_kl(const spec_attn_args_t& a, const AttnPlan& P, char* ws,
                            cudaStream_t stream);
 cudaError_t launch_philox(uint64_t seed, uint64_t offset, int64_t n, float* out, cudaStream_t s);

@@ -175,3 +175,77 @@ def test_deterministic_repeat():
     out1, lse1 = binding.verify_attention(*t)
     out2, lse2 = binding.verify_attention(*t)
     assert torch.equal(out1, out2) and torch.equal(lse1, lse2)
+
+
+# The small-group kernel (automatic choice): 1 to 64 query rows per KV head (edges of its
+# 16-row tiles), 2, 4 and 8 KV heads per block, every page size, contexts that end inside
+# a 16-key step, units whole in a block, split over a few blocks and over many.
+GROUPS = [
+    dict(batch=1, gamma=1, num_q_heads=2, num_kv_heads=2, head_dim=128, page_size=16, ctx=0),
+    dict(batch=24, gamma=1, num_q_heads=32, num_kv_heads=8, head_dim=128, page_size=16, ctx=(0, 900)),
+    dict(batch=1, gamma=1, num_q_heads=8, num_kv_heads=8, head_dim=64, page_size=32, ctx=6000),
+    dict(batch=20, gamma=3, num_q_heads=40, num_kv_heads=8, head_dim=128, page_size=32, ctx=(5, 700)),
+    dict(batch=3, gamma=4, num_q_heads=16, num_kv_heads=4, head_dim=128, page_size=64, ctx=(100, 2000)),
+    dict(batch=40, gamma=16, num_q_heads=8, num_kv_heads=8, head_dim=128, page_size=16, ctx=(1, 300)),
+    dict(batch=5, gamma=17, num_q_heads=6, num_kv_heads=6, head_dim=128, page_size=16, ctx=(60, 700)),
+    dict(batch=40, gamma=8, num_q_heads=16, num_kv_heads=4, head_dim=128, page_size=64, ctx=(1, 500)),
+    dict(batch=7, gamma=11, num_q_heads=12, num_kv_heads=4, head_dim=128, page_size=16, ctx=(0, 333)),
+    dict(batch=2, gamma=48, num_q_heads=2, num_kv_heads=2, head_dim=128, page_size=32, ctx=(0, 1500)),
+    dict(batch=30, gamma=49, num_q_heads=4, num_kv_heads=4, head_dim=64, page_size=16, ctx=(0, 400)),
+    dict(batch=9, gamma=64, num_q_heads=8, num_kv_heads=8, head_dim=64, page_size=64, ctx=(3, 900)),
+    dict(batch=50, gamma=2, num_q_heads=32, num_kv_heads=8, head_dim=64, page_size=16, ctx=(0, 500)),
+    dict(batch=300, gamma=2, num_q_heads=4, num_kv_heads=2, head_dim=128, page_size=16, ctx=(0, 90)),
+]
+
+
+@pytest.mark.parametrize("case", range(len(GROUPS)))
+def test_small_groups(oracle_mod, case):
+    inp = W.make_attn_inputs(seed=200 + case, **GROUPS[case])
+    g_out, g_lse = gpu_attention(inp, binding.ATTN_AUTO)
+    o_out, o_lse, st = oracle_attn(oracle_mod, inp)
+    assert np.all(st == 0)
+    compare_attention(g_out, g_lse, o_out, o_lse)
+
+
+@pytest.mark.parametrize("case", [0, 2, 3, 6, 9])
+def test_small_groups_tree_mask(oracle_mod, case):
+    inp = W.make_attn_inputs(seed=230 + case, **GROUPS[case])
+    B, N = inp.batch, inp.gamma
+    rng = np.random.default_rng(case)
+    masks = np.zeros((B, N), np.uint64)
+    for b in range(B):
+        for j in range(N):
+            up = masks[b, int(rng.integers(0, j))] if j else np.uint64(0)
+            masks[b, j] = up | np.uint64(1 << j)
+    out, lse = binding.verify_attention(*attn_tensors(inp), tree_mask=torch.from_numpy(masks.view(np.int64)).cuda())
+    o_out, o_lse, st = oracle_mod.verify_attention(inp.q, inp.k_cache, inp.v_cache, inp.page_table,
+                                                   inp.kv_len, N, tree_mask=masks)
+    assert np.all(st == 0)
+    compare_attention(out.float().cpu().numpy(), lse.cpu().numpy(), o_out, o_lse)
+
+
+@pytest.mark.parametrize("gamma,head_dim,page", [(1, 128, 16), (8, 128, 32), (4, 64, 64), (16, 128, 16)])
+def test_small_groups_bad_inputs_and_garbage(oracle_mod, gamma, head_dim, page):
+    inp = W.make_attn_inputs(5, gamma, 16, 4, head_dim, page, (150, 400), seed=240 + gamma)
+    inp.page_table[1, 2] = inp.num_pages + 5
+    inp.page_table[4, int(inp.kv_len[4] - 1) // page] = -3
+    inp.kv_len[2] = inp.page_table.shape[1] * page + 1  # longer than its pages
+    for b in (0, 3):  # NaN in the unused tail of the last page
+        L = int(inp.kv_len[b])
+        last = inp.page_table[b, (L - 1) // page]
+        if L % page:
+            inp.k_cache[last, :, L % page:] = 0x7FC0
+            inp.v_cache[last, :, L % page:] = 0x7FC0
+    t = attn_tensors(inp)
+    out = torch.empty_like(t[0])
+    lse = torch.empty(t[0].shape[:3], dtype=torch.float32, device="cuda")
+    a = binding.attn_args(*t, out, lse)
+    ws = binding.new_workspace(binding.workspace_size(attn=a))
+    for _ in range(2):  # the workspace serves the next call
+        out.fill_(1.0)
+        binding.verify_attention_args(a, ws)
+        code, flags = binding.read_device_status(ws)
+        assert code == 5 and flags == (binding.FLAG_BAD_PAGE | binding.FLAG_BAD_KV_LEN)
+        o_out, o_lse, st = oracle_attn(oracle_mod, inp)
+        assert list(st) == [0, 1, 1, 0, 1]
+        compare_attention(out.float().cpu().numpy(), lse.cpu().numpy(), o_out, o_lse)
