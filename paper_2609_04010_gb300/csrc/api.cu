@@ -312,8 +312,12 @@ AttnPlan attn_plan(const spec_attn_args_t& a, size_t base, int num_sms, int path
     P.slot_rows = (P.rows < P.rows_per_cta ? P.rows : P.rows_per_cta) * (1 + P.head_pair);
     P.slots = units + P.grid;
   }
+  // every path's counters lie in the same region (that of the path with the most units, the
+  // CUDA-core kernel), ahead of any scratch data: the paths may take turns on a workspace
   P.tickets = base;
-  P.partial_o = ws_round(P.tickets + sizeof(uint32_t) * units);
+  P.splits = ws_round(P.tickets + sizeof(uint32_t) * static_cast<size_t>(a.batch) * a.num_kv_heads *
+                                      ((P.rows + kSimtRowTile - 1) / kSimtRowTile));
+  P.partial_o = ws_round(P.splits + sizeof(SplitUnit) * P.grid);
   P.partial_ml =
       ws_round(P.partial_o + static_cast<size_t>(P.slots) * P.slot_rows * a.head_dim * 4);
   P.end = ws_round(P.partial_ml + static_cast<size_t>(P.slots) * P.slot_rows * sizeof(float2));

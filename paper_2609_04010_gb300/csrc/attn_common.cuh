@@ -31,6 +31,7 @@ struct AttnParams {
   float* lse;
   uint32_t* status;
   uint32_t* tickets;
+  SplitUnit* splits;   // [grid]
   float* partial_o;    // [slot][slot_rows][D]
   float2* partial_ml;  // [slot][slot_rows] = (m, l); l = -1 marks a bad sequence
   int q_tma;           // tensor-core kernel: Q tiles arrive by TMA (else softmax warps load them)
@@ -70,6 +71,7 @@ inline AttnParams make_attn_params(const spec_attn_args_t& a, const AttnPlan& P,
   p.lse = a.lse;
   p.status = reinterpret_cast<uint32_t*>(ws);
   p.tickets = reinterpret_cast<uint32_t*>(ws + P.tickets);
+  p.splits = reinterpret_cast<SplitUnit*>(ws + P.splits);
   p.partial_o = reinterpret_cast<float*>(ws + P.partial_o);
   p.partial_ml = reinterpret_cast<float2*>(ws + P.partial_ml);
   p.q_tma = 0;
@@ -270,198 +272,201 @@ __device__ void merge_unit(const AttnParams& p, int b, int g, int row0, int nrow
   }
 }
 
-// Contiguous global -> shared copy by the copy engine, completing on bar (16-byte aligned
-// addresses, size a multiple of 16).
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-               "l"(src), "r"(bytes), "r"(bar)
-               : "memory");
-}
-// Orders this thread's view of global memory (generic proxy) before its later copies
-// by the copy engine (async proxy).
-__device__ __forceinline__ void fence_async_global() {
-  asm volatile("fence.proxy.async.global;" ::: "memory");
-}
-
-// Merge of one unit from its partial slots staged in shared memory: so[nsl][slot_rows][D]
-// and sml[nsl][slot_rows] = (m, l), row r of [row0, row0 + nrows) at slot row prow0 + r.
-// The same combination as merge_unit, with every load from shared memory.
-template <int D>
-__device__ void merge_staged(const AttnParams& p, int b, int g, int row0, int nrows, const float* so,
-                             const float2* sml, int nsl, int prow0, int tid, int nthreads) {
-  constexpr int C8 = D / 8;
-  for (int idx = tid; idx < nrows * C8; idx += nthreads) {
-    const int r = idx / C8, c8 = idx % C8, pr = prow0 + r;
-    float mx = -INFINITY;
-    bool bad = false;
-    for (int i = 0; i < nsl; ++i) {
-      const float2 ml = sml[i * p.slot_rows + pr];
-      bad |= ml.y < 0.f;
-      if (ml.y > 0.f) mx = fmaxf(mx, ml.x);
-    }
-    float L = 0.f, acc[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) acc[e] = 0.f;
-    if (mx != -INFINITY) {
-      for (int i = 0; i < nsl; ++i) {
-        const float2 ml = sml[i * p.slot_rows + pr];
-        if (!(ml.y > 0.f)) continue;
-        const float w = ex2(ml.x - mx);
-        const float4* src = reinterpret_cast<const float4*>(so + (static_cast<size_t>(i) * p.slot_rows + pr) * D) + 2 * c8;
-        const float4 a = src[0], c = src[1];
-        L += ml.y * w;
-        acc[0] += a.x * w; acc[1] += a.y * w; acc[2] += a.z * w; acc[3] += a.w * w;
-        acc[4] += c.x * w; acc[5] += c.y * w; acc[6] += c.z * w; acc[7] += c.w * w;
-      }
-    }
-    const bool dead = bad || !(L > 0.f);
-    write_out_row<D>(p, b, g, row0 + r, c8 * 8, acc, dead ? 0.f : 1.f / L);
-    if (c8 == 0) write_lse(p, b, g, row0 + r, mx, L, dead);
-  }
-}
-
 // ---------------------------------------------------------------------------------
 // Merging split units in a kernel of their own
 // ---------------------------------------------------------------------------------
-// pb[b] = virtual tiles of the sequences before b (one warp).
+// pb[b] = virtual tiles of the sequences before b (one warp, four sequences a lane and round:
+// each round's loads are one trip to memory).
 template <int TK>
 __device__ __forceinline__ void tile_prefix(const AttnParams& p, int* pb, int lane) {
   const int per_b = p.hunits * p.row_tiles;
   int carry = 0;
-  for (int b0 = 0; b0 < p.batch; b0 += 32) {
-    const int b = b0 + lane;
-    int v = b < p.batch ? (unit_tiles<TK>(p.kv_len[b], p) + p.unit_overhead) * per_b : 0;
+  for (int b0 = 0; b0 < p.batch; b0 += 128) {
+    int v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int b = b0 + 4 * lane + i;
+      v[i] = b < p.batch ? p.kv_len[b] : 0;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      v[i] = (b0 + 4 * lane + i < p.batch ? (unit_tiles<TK>(v[i], p) + p.unit_overhead) * per_b : 0) + (i > 0 ? v[i - 1] : 0);
+    int sum = v[3];
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, v, o);
-      if (lane >= o) v += y;
+      const int y = __shfl_up_sync(0xffffffffu, sum, o);
+      if (lane >= o) sum += y;
     }
-    if (b < p.batch) pb[b + 1] = carry + v;
-    carry += __shfl_sync(0xffffffffu, v, 31);
+    const int before = carry + sum - v[3];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (b0 + 4 * lane + i < p.batch) pb[b0 + 4 * lane + i + 1] = before + v[i];
+    carry += __shfl_sync(0xffffffffu, sum, 31);
   }
   if (lane == 0) pb[0] = 0;
 }
 
 // Ranges the virtual tiles are cut into: one per block, of at least min_tiles tiles each
 // (below that a block's start, partial and merge cost more than the tiles it takes off the
-// others).
+// others). Every SM gets a range: with the merges in a kernel of their own, 32 equal units
+// over all 152 blocks take less time than over 128 blocks of a quarter unit each (4 sequences
+// of 32,768 keys, 256 rows per KV head: 161 us against 182).
 __device__ __forceinline__ int range_count(int64_t total, const AttnParams& p) {
   const int64_t want = (total + p.min_tiles - 1) / p.min_tiles;
   return want < p.grid ? static_cast<int>(want) : p.grid;
 }
 
-// The outputs of the units that were split between blocks, from their partial slots. Block
-// (c, y) stands for the boundary before range c + 1: the k-th boundary inside a unit merges
-// the k-th share of the unit's rows (of gridDim.y pieces, piece y), so that every block
-// reads about one slot however many ways a unit was split. One warp takes a row at a time;
-// its loads of all slots are in flight together. Merging in the last block of a unit to
-// finish instead (atomic ticket) left most SMs idle while a few read every slot: 3 us for
-// the fence and the ticket and 7 to 15 us for the merge (8 requests of 32 rows per KV head
-// and 4,096 keys: 53.3 us; here 37.2).
-constexpr int kAttnMergeThreads = 256;
-constexpr int kAttnMergePieces = 2;
-template <int D, int TK>
-__global__ void __launch_bounds__(kAttnMergeThreads) attn_merge_kernel(AttnParams p) {
-  extern __shared__ int pb_sh[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (warp == 0) tile_prefix<TK>(p, pb_sh, lane);
-  __syncthreads();
-  const int64_t total = pb_sh[p.batch];
-  const int ctas = range_count(total, p);
-  const int c = blockIdx.x + 1;
-  if (c >= ctas) return;
-  const Seg s = locate<TK>(static_cast<int64_t>(c) * total / ctas, total, p, pb_sh, p.unit_overhead);
-  // the boundary lies inside the unit's real tiles
-  if (static_cast<int64_t>(c) * total / ctas <= s.unit_start) return;
-  const int c_first = owner_of(s.unit_start, total, ctas);
-  const int nsl = owner_of(s.unit_start + s.unit_tiles - 1, total, ctas) - c_first + 1;
-  const int rows = min(p.slot_rows, p.unit_heads * min(p.rows_per_cta, p.rows - s.rt * p.rows_per_cta));
-  const int parts = (nsl - 1) * gridDim.y, part = (c - c_first - 1) * gridDim.y + blockIdx.y;
-  const int r_end = static_cast<int>(static_cast<int64_t>(rows) * (part + 1) / parts);
-  const int head_rows = rows / p.unit_heads;  // a unit's heads follow each other in a slot
-  const int64_t slot0 = s.u + c_first;
+// What the merge kernel reads of block cta's left boundary, s its first segment (one thread).
+__device__ __forceinline__ void note_split(const AttnParams& p, int cta, const Seg& s, int64_t total, int ctas) {
+  SplitUnit d = {};
+  if (s.ntile > 0 && s.tile0 > 0) {
+    const int c_first = owner_of(s.unit_start, total, ctas);
+    d.b = s.b;
+    d.g = s.g;
+    d.rt = s.rt;
+    d.slot0 = static_cast<int>(s.u) + c_first;
+    d.nsl = owner_of(s.unit_start + s.unit_tiles - 1, total, ctas) - c_first + 1;
+    d.k = cta - c_first - 1;
+  }
+  p.splits[cta] = d;
+}
+
+// RW rows of one warp from their partial slots [slot0, slot0 + nsl), SB slots at a time: the
+// loads of all those rows and slots are in flight together.
+template <int D, int RW, int SB>
+__device__ __forceinline__ void merge_rows(const AttnParams& p, const SplitUnit& u, int r0, int r_end,
+                                           int head_rows, int lane) {
   constexpr int E = D / 32;  // output columns per lane
-  constexpr int SB = 8;      // slots whose loads are in flight together
-  pdl_wait_prior();
-  for (int r = static_cast<int>(static_cast<int64_t>(rows) * part / parts) + warp; r < r_end;
-       r += kAttnMergeThreads / 32) {
-    float M = -INFINITY, L = 0.f, acc[E];
-    bool bad = false;
+  float M[RW], L[RW], acc[RW][E];
+  bool bad[RW];
 #pragma unroll
-    for (int e = 0; e < E; ++e) acc[e] = 0.f;
-    for (int s0 = 0; s0 < nsl; s0 += SB) {
-      float2 ml[SB];
-      float o[SB][E];
+  for (int t = 0; t < RW; ++t) {
+    M[t] = -INFINITY;
+    L[t] = 0.f;
+    bad[t] = false;
+#pragma unroll
+    for (int e = 0; e < E; ++e) acc[t][e] = 0.f;
+  }
+  for (int s0 = 0; s0 < u.nsl; s0 += SB) {
+    float2 ml[RW][SB];
+    float o[RW][SB][E];
+#pragma unroll
+    for (int t = 0; t < RW; ++t)
 #pragma unroll
       for (int i = 0; i < SB; ++i) {
-        const int64_t row = (slot0 + s0 + i) * p.slot_rows + r;
-        ml[i] = make_float2(-INFINITY, 0.f);
+        ml[t][i] = make_float2(-INFINITY, 0.f);
 #pragma unroll
-        for (int e = 0; e < E; ++e) o[i][e] = 0.f;
-        if (s0 + i < nsl) {
-          ml[i] = __ldcg(&p.partial_ml[row]);
-          if (E == 4) {
+        for (int e = 0; e < E; ++e) o[t][i][e] = 0.f;
+        if (r0 + t < r_end && s0 + i < u.nsl) {
+          const int64_t row = static_cast<int64_t>(u.slot0 + s0 + i) * p.slot_rows + r0 + t;
+          ml[t][i] = __ldcg(&p.partial_ml[row]);
+          if constexpr (E == 4) {
             const float4 v = __ldcg(reinterpret_cast<const float4*>(p.partial_o + row * D) + lane);
-            o[i][0] = v.x; o[i][1] = v.y; o[i][E - 2] = v.z; o[i][E - 1] = v.w;
+            o[t][i][0] = v.x; o[t][i][1] = v.y; o[t][i][2] = v.z; o[t][i][3] = v.w;
           } else {
             const float2 v = __ldcg(reinterpret_cast<const float2*>(p.partial_o + row * D) + lane);
-            o[i][0] = v.x; o[i][1] = v.y;
+            o[t][i][0] = v.x; o[t][i][1] = v.y;
           }
         }
       }
-      float mb = M;
+#pragma unroll
+    for (int t = 0; t < RW; ++t) {
+      float mb = M[t];
 #pragma unroll
       for (int i = 0; i < SB; ++i) {
-        bad |= ml[i].y < 0.f;
-        if (ml[i].y > 0.f) mb = fmaxf(mb, ml[i].x);
+        bad[t] |= ml[t][i].y < 0.f;
+        if (ml[t][i].y > 0.f) mb = fmaxf(mb, ml[t][i].x);
       }
       if (mb == -INFINITY) continue;
-      const float scale = M == -INFINITY ? 0.f : ex2(M - mb);
-      L *= scale;
+      const float scale = M[t] == -INFINITY ? 0.f : ex2(M[t] - mb);
+      L[t] *= scale;
 #pragma unroll
-      for (int e = 0; e < E; ++e) acc[e] *= scale;
+      for (int e = 0; e < E; ++e) acc[t][e] *= scale;
 #pragma unroll
       for (int i = 0; i < SB; ++i) {
-        if (!(ml[i].y > 0.f)) continue;
-        const float w = ex2(ml[i].x - mb);
-        L += ml[i].y * w;
+        if (!(ml[t][i].y > 0.f)) continue;
+        const float w = ex2(ml[t][i].x - mb);
+        L[t] += ml[t][i].y * w;
 #pragma unroll
-        for (int e = 0; e < E; ++e) acc[e] += o[i][e] * w;
+        for (int e = 0; e < E; ++e) acc[t][e] += o[t][i][e] * w;
       }
-      M = mb;
+      M[t] = mb;
     }
-    const bool dead = bad || !(L > 0.f);
-    const float inv = dead ? 0.f : 1.f / L;
-    const int kvh = s.g * p.unit_heads + r / head_rows, row = s.rt * p.rows_per_cta + r % head_rows;
+  }
+#pragma unroll
+  for (int t = 0; t < RW; ++t) {
+    const int r = r0 + t;
+    if (r >= r_end) break;
+    const bool dead = bad[t] || !(L[t] > 0.f);
+    const float inv = dead ? 0.f : 1.f / L[t];
+    const int kvh = u.g * p.unit_heads + r / head_rows, row = u.rt * p.rows_per_cta + r % head_rows;
     const int j = row / p.group, h = kvh * p.group + row % p.group;
     uint32_t w[E / 2];
 #pragma unroll
     for (int e = 0; e < E / 2; ++e) {
-      const __nv_bfloat162 v = __floats2bfloat162_rn(dead ? 0.f : acc[2 * e] * inv, dead ? 0.f : acc[2 * e + 1] * inv);
+      const __nv_bfloat162 v = __floats2bfloat162_rn(dead ? 0.f : acc[t][2 * e] * inv, dead ? 0.f : acc[t][2 * e + 1] * inv);
       w[e] = *reinterpret_cast<const uint32_t*>(&v);
     }
     __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(p.out) +
-                         ((static_cast<int64_t>(s.b) * p.gamma + j) * p.hq + h) * D + lane * E;
-    if (E == 4) *reinterpret_cast<uint2*>(dst) = make_uint2(w[0], w[E / 2 - 1]);
+                         ((static_cast<int64_t>(u.b) * p.gamma + j) * p.hq + h) * D + lane * E;
+    if constexpr (E == 4) *reinterpret_cast<uint2*>(dst) = make_uint2(w[0], w[1]);
     else *reinterpret_cast<uint32_t*>(dst) = w[0];
-    if (lane == 0) write_lse(p, s.b, kvh, row, M, L, dead);
+    if (lane == 0) write_lse(p, u.b, kvh, row, M[t], L[t], dead);
   }
 }
 
-template <int D, int TK>
+// The outputs of the units that were split between blocks, from their partial slots. Block
+// (c, y) stands for the boundary before range c + 1: the k-th boundary inside a unit merges
+// the k-th share of the unit's rows (of gridDim.y pieces, piece y), so that every boundary
+// reads about one slot however many ways a unit was split (the blocks leave the boundaries'
+// descriptions behind; finding them from the lengths again was 1 us slower). Merging in the last block of a
+// unit to finish instead (atomic ticket) left most SMs idle while a few read every slot:
+// 3 us for the fence and the ticket and 7 to 15 us for the merge (one request of 128 rows per
+// KV head and 4,096 keys: 46.7 us, here 18.6; 8 requests of 32 rows: 53, here 38; 64 ragged
+// requests of 64 rows: 124.0, here 118.2).
+constexpr int kAttnMergeThreads = 256;
+template <int D>
+__global__ void __launch_bounds__(kAttnMergeThreads) attn_merge_kernel(AttnParams p) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  pdl_wait_prior();
+  const int4 lo = __ldcg(reinterpret_cast<const int4*>(p.splits + blockIdx.x + 1));
+  const int4 hi = __ldcg(reinterpret_cast<const int4*>(p.splits + blockIdx.x + 1) + 1);
+  SplitUnit u;
+  u.b = lo.x;
+  u.g = lo.y;
+  u.rt = lo.z;
+  u.slot0 = lo.w;
+  u.nsl = hi.x;
+  u.k = hi.y;
+  if (u.nsl < 2) return;
+  // a unit's heads follow each other in a slot
+  const int head_rows = min(p.rows_per_cta, p.rows - u.rt * p.rows_per_cta), rows = p.unit_heads * head_rows;
+  const int parts = (u.nsl - 1) * gridDim.y, part = u.k * gridDim.y + blockIdx.y;
+  const int r_begin = static_cast<int>(static_cast<int64_t>(rows) * part / parts);
+  const int r_end = static_cast<int>(static_cast<int64_t>(rows) * (part + 1) / parts);
+  constexpr int W = kAttnMergeThreads / 32;
+  if (u.nsl == 2) {
+    for (int r = r_begin + 4 * warp; r < r_end; r += 4 * W) merge_rows<D, 4, 2>(p, u, r, r_end, head_rows, lane);
+  } else {
+    for (int r = r_begin + warp; r < r_end; r += W) merge_rows<D, 1, 8>(p, u, r, r + 1, head_rows, lane);
+  }
+}
+
+template <int D>
 cudaError_t launch_merge(const AttnParams& p, cudaStream_t stream) {
   if (p.grid < 2) return cudaSuccess;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(p.grid - 1, kAttnMergePieces);
+  // Two blocks per boundary are one wave of them, and one pass of their warps over the rows
+  // of a two-slot unit of up to 128 rows (four per boundary, two waves: 2 to 3 us slower).
+  cfg.gridDim = dim3(p.grid - 1, p.slot_rows <= 32 ? 1 : 2);
   cfg.blockDim = dim3(kAttnMergeThreads);
-  cfg.dynamicSmemBytes = 4u * (p.batch + 1);
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, attn_merge_kernel<D, TK>, p);
+  return cudaLaunchKernelEx(&cfg, attn_merge_kernel<D>, p);
 }
 #endif
 

@@ -166,7 +166,8 @@ __global__ void __launch_bounds__(MmaCfg<D, HB, MTW>::THREADS, 1)
     const CUtensorMap* map = warp == 0 ? &tmap_k : &tmap_v;
     const uint32_t ring = sbase + (warp == 0 ? 0u : C::OFF_V);
     const uint32_t box_bytes = static_cast<uint32_t>(box_keys) * D * 2 * HB;
-    for (Seg s = locate<KS>(t0, t1, p, pb, OVH); s.ntile > 0 && ok;) {
+    const Seg s_first = locate<KS>(t0, t1, p, pb, OVH);
+    for (Seg s = s_first; s.ntile > 0 && ok;) {
       for (int k = 0; k < s.ntile; ++k, ++it) {
         const uint32_t st = it % S;
         if (it >= S) ok = mbar_wait(empty(st), ((it / S) - 1) & 1, abort_flag, p.status);
@@ -199,6 +200,10 @@ __global__ void __launch_bounds__(MmaCfg<D, HB, MTW>::THREADS, 1)
       if (!ok || !has_more(s, t1, OVH)) break;
       s = locate<KS>(s.vnext, t1, p, pb, OVH);
     }
+    // the block's last tiles are on their way: the merge kernel's blocks may be brought in
+    // (they wait for the whole grid, and find room only where a block has ended)
+    if (warp == 1 && lane == 0) note_split(p, cta, s_first, total, ctas);
+    pdl_launch_dependents();
     if (!ok) {  // copies still in flight land before the block exits (bounded)
       for (uint32_t x = it > S ? it - S : 0; x < it; ++x) {
         const long long c0 = clock64();
@@ -499,9 +504,6 @@ __global__ void __launch_bounds__(MmaCfg<D, HB, MTW>::THREADS, 1)
       s = locate<KS>(s.vnext, t1, p, pb, OVH);
     }
   }
-  // every partial of the block is written: the merge kernel may be brought in (it waits for
-  // the whole grid before it reads them)
-  pdl_launch_dependents();
 }
 
 // ---------------------------------------------------------------------------------
@@ -547,7 +549,7 @@ cudaError_t launch_typed(const spec_attn_args_t& a, const AttnPlan& P, char* ws,
   if (e != cudaSuccess) return e;
   kernel<<<P.grid, C::THREADS, smem, stream>>>(mk, mv, p, box_keys);
   const cudaError_t launched = cudaGetLastError();
-  return launched != cudaSuccess ? launched : launch_merge<D, C::KS>(p, stream);
+  return launched != cudaSuccess ? launched : launch_merge<D>(p, stream);
 }
 
 template <int D, int HB>

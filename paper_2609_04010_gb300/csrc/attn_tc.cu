@@ -39,9 +39,8 @@
 //               write the output. Warps without real rows idle.
 // Work is balanced across blocks "stream-K" style: all 64-key tiles of all (sequence,
 // KV head, row tile) units form one list that is cut into equal contiguous ranges; a
-// unit split between blocks is merged from fp32 partials by the last block to finish
-// it (atomic ticket, no waiting; a head pair's slots are first brought into the idle
-// K/V stages by bulk copies). Every mbarrier wait is bounded: a wait that runs out
+// unit split between blocks is merged from fp32 partials by attn_merge_kernel
+// (attn_common.cuh). Every mbarrier wait is bounded: a wait that runs out
 // sets SPEC_FLAG_TIMEOUT, drains the block's own copies and MMAs, frees TMEM and exits.
 #include <cuda.h>  // CUtensorMap and its encoder's signature (resolved at run time)
 
@@ -99,17 +98,13 @@ struct TcCfg {
   static constexpr uint32_t OFF_K = QR == 64 ? OFF_P + P_BYTES : OFF_Q + Q_BYTES;
   static constexpr uint32_t OFF_V = OFF_K + KST * KV_BYTES;
   static constexpr uint32_t OFF_BAR = QR == 64 ? OFF_V + VST * KV_BYTES : OFF_P + P_BYTES;
-  // the K and V stages, contiguous from OFF_K; at a block's end they stage the partials
-  // of the units it merges
-  static constexpr uint32_t RING_BYTES = (KST + VST) * KV_BYTES;
   // barriers: ring (kv_full[S], kv_empty[S], or k_full[KST], v_full[VST], k_empty[KST],
   // v_empty[VST]), s_full[MT][2], s_free[MT][2], p_full[MT][PB], pv_done[MT][PB],
-  // seg_ready, drain[2], xch[4], q_full, seg_flag_ready[8], merge_staged (HP = 2)
-  static constexpr int NBAR = RINGBARS + 4 * MT + 2 * MT * PB + 3 + 4 + 1 + 8 + (HP == 2 ? 1 : 0);
-  static constexpr uint32_t OFF_MISC = OFF_BAR + NBAR * 8;  // tmem base, abort, pending count
+  // seg_ready, drain[2], xch[4], q_full, seg_flag_ready[8]
+  static constexpr int NBAR = RINGBARS + 4 * MT + 2 * MT * PB + 3 + 4 + 1 + 8;
+  static constexpr uint32_t OFF_MISC = OFF_BAR + NBAR * 8;  // tmem base, abort flag
   static constexpr uint32_t OFF_XCH = OFF_MISC + 16;        // [4][2][32] float2 (m, l) per half
-  static constexpr uint32_t OFF_PEND = OFF_XCH + (SPLIT == 2 ? 4 * 2 * 32 * 8 : 0);  // [2][8]
-  static constexpr uint32_t OFF_FLAG = OFF_PEND + 64;  // [8] bad flags of segments
+  static constexpr uint32_t OFF_FLAG = OFF_XCH + (SPLIT == 2 ? 4 * 2 * 32 * 8 : 0);  // [8] bad flags of segments
   static constexpr uint32_t OFF_PB = (OFF_FLAG + 32 + 15) / 16 * 16;
   // accumulators a = mt * HP + head: S[a][buf] at (a * 2 + buf) * 64, O[a][half] at
   // O_COL + (a * SPLIT + half) * D
@@ -195,18 +190,12 @@ __global__ void __launch_bounds__(TcCfg<D, MT, QR, HP>::THREADS, 1)
   // segment flags: the producer publishes whether a segment reads a bad page or has a
   // malformed length (ring of 8, far more than the producer can run ahead)
   auto flag_bar = [&](int i) { return seg_ready + 64 + 8u * i; };
-  const uint32_t merge_bar = seg_ready + 128;  // a unit's partials staged in the ring
   volatile int* seg_flag = reinterpret_cast<volatile int*>(smem + C::OFF_FLAG);
   uint32_t* misc = reinterpret_cast<uint32_t*>(smem + C::OFF_MISC);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 1);
-  volatile int* pend_count = reinterpret_cast<volatile int*>(misc + 2);
-  // split units this block wrote partials for (only a block's first and last segments
-  // can be split): b, g, row0, nrows, first slot, slots, unit, merge-here flag
-  int* pend = reinterpret_cast<int*>(smem + C::OFF_PEND);
   int* pb = reinterpret_cast<int*>(smem + C::OFF_PB);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  pdl_launch_dependents();  // the acceptance kernels of a verify step may start beside us
 
   // ---- roles ----
   // Softmax warps take part only as far as the row tile has real rows (32 per warp).
@@ -261,46 +250,18 @@ __global__ void __launch_bounds__(TcCfg<D, MT, QR, HP>::THREADS, 1)
     for (int q = 0; q < 4; ++q) mbar_init(xch_bar(q), 2);
     mbar_init(q_full, 1);
     for (int i = 0; i < 8; ++i) mbar_init(flag_bar(i), 1);
-    if (HP == 2) mbar_init(merge_bar, 1);
     *abort_flag = 0;
-    *pend_count = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) tmem_alloc(smem_u32(misc), C::TMEM_COLS);
-  if (warp == 0) {
-    const int per_b = p.hunits * p.row_tiles;
-    int carry = 0;
-    for (int b0 = 0; b0 < p.batch; b0 += 32) {
-      const int b = b0 + lane;
-      int v = b < p.batch ? (unit_tiles<TK>(p.kv_len[b], p) + p.unit_overhead) * per_b : 0;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += y;
-      }
-      if (b < p.batch) pb[b + 1] = carry + v;
-      carry += __shfl_sync(0xffffffffu, v, 31);
-    }
-    if (lane == 0) pb[0] = 0;
-  }
+  if (warp == 0) tile_prefix<TK>(p, pb, lane);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = misc[0];
 
   const int64_t total = pb[p.batch];
-  // With no more units than blocks, use a multiple of the unit count: equal-length
-  // units then split into equal parts with no unit boundary inside any block's range
-  // (a few SMs idle; measured faster than spreading boundaries and extra merges over
-  // every SM). Ranges stay equal in tiles, so ragged lengths stay balanced.
-  int ctas = static_cast<int>(total < gridDim.x ? total : gridDim.x);
-  {
-    const int units = p.batch * p.hunits * p.row_tiles;
-    if (units <= static_cast<int>(gridDim.x)) {
-      const int aligned = units * (static_cast<int>(gridDim.x) / units);
-      if (aligned < ctas) ctas = aligned;
-    }
-  }
+  const int ctas = range_count(total, p);
   const int cta = blockIdx.x;
   const int64_t t0 = cta < ctas ? static_cast<int64_t>(cta) * total / ctas : 0;
   const int64_t t1 = cta < ctas ? static_cast<int64_t>(cta + 1) * total / ctas : 0;
@@ -337,7 +298,8 @@ __global__ void __launch_bounds__(TcCfg<D, MT, QR, HP>::THREADS, 1)
     const uint32_t ring_base = sbase + (pw == 0 ? C::OFF_K : C::OFF_V);
     const CUtensorMap* map = pw == 0 ? &tmap_k : &tmap_v;
     uint32_t seg_no = 0;
-    for (Seg s = locate<TK>(t0, t1, p, pb, OVH); s.ntile > 0 && ok && !p.starve; ++seg_no) {
+    const Seg s_first = locate<TK>(t0, t1, p, pb, OVH);
+    for (Seg s = s_first; s.ntile > 0 && ok && !p.starve; ++seg_no) {
       const bool bad = !s.len_ok;  // nothing to read
       bool flag = bad;             // ... or a page id out of range (read as page 0)
       for (int k = 0; k < s.ntile && ok; ++k, ++it) {
@@ -371,6 +333,10 @@ __global__ void __launch_bounds__(TcCfg<D, MT, QR, HP>::THREADS, 1)
       if (!has_more(s, t1, OVH)) break;
       s = locate<TK>(s.vnext, t1, p, pb, OVH);
     }
+    // the block's last tiles are on their way: the merge kernel's blocks may be brought in
+    // (they wait for the whole grid, and find room only where a block has ended)
+    if (warp == 2 && lane == 0) note_split(p, cta, s_first, total, ctas);
+    pdl_launch_dependents();
     if (!ok) {  // drain this producer's copies still in flight (bounded)
       for (uint32_t x = it > RS ? it - RS : 0; x < it; ++x) {
         const long long t_0 = clock64();
@@ -747,10 +713,8 @@ __global__ void __launch_bounds__(TcCfg<D, MT, QR, HP>::THREADS, 1)
         L = l0 * sc0 + l1 * sc1;
       }
       const bool whole = s.tile0 == 0 && s.ntile == s.unit_tiles;
-      const int c_first = owner_of(s.unit_start, total, ctas);
-      const int c_last = owner_of(s.unit_start + s.unit_tiles - 1, total, ctas);
       const int64_t slot = s.u + cta;
-      if (bad && sw == 0 && lane == 0 && (whole || cta == c_first))
+      if (bad && sw == 0 && lane == 0)
         set_status(p.status, s.len_ok ? SPEC_FLAG_BAD_PAGE : SPEC_FLAG_BAD_KV_LEN);
       // this warp writes output columns [hf * D / SPLIT, (hf + 1) * D / SPLIT)
 #pragma unroll 1
@@ -789,15 +753,6 @@ __global__ void __launch_bounds__(TcCfg<D, MT, QR, HP>::THREADS, 1)
         if (whole) write_lse(p, s.b, ro.kvh, ro.urow, M, L, bad);
         else p.partial_ml[slot * p.slot_rows + prow] = make_float2(M, bad ? -1.f : L);
       }
-      if (!whole && sw == 0 && lane == 0) {
-        // the ticket of a split unit is taken at the end of the block, after a fence
-        int* e = pend + 8 * (*pend_count);
-        const int row0 = s.rt * p.rows_per_cta;
-        e[0] = s.b; e[1] = s.g; e[2] = row0; e[3] = min(p.rows_per_cta, p.rows - row0);
-        e[4] = static_cast<int>(s.u + c_first); e[5] = c_last - c_first + 1;
-        e[6] = static_cast<int>(s.u); e[7] = 0;
-        *pend_count = *pend_count + 1;
-      }
       it += s.ntile;
       s = sn;
       ++seg_no;
@@ -808,72 +763,6 @@ __global__ void __launch_bounds__(TcCfg<D, MT, QR, HP>::THREADS, 1)
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, C::TMEM_COLS);
-  }
-  // Split units: every thread makes its partial writes visible, then the block takes
-  // one ticket per unit it wrote; the block that completes a unit merges it.
-  if (!*abort_flag) {
-    const int np = *pend_count;  // block-uniform
-    if (np > 0) {
-      __threadfence();
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        for (int i = 0; i < np; ++i) {
-          int* e = pend + 8 * i;
-          const uint32_t prev = atomicAdd(&p.tickets[e[6]], 1u);
-          e[7] = prev == static_cast<uint32_t>(e[5] - 1);
-          if (e[7]) p.tickets[e[6]] = 0;  // leave the counter at zero for the next call
-        }
-      }
-      __syncthreads();
-      bool any = false;
-      for (int i = 0; i < np; ++i) any |= pend[8 * i + 7] != 0;
-      if (any) __threadfence();
-      uint32_t mphase = 0;
-      for (int i = 0; i < np; ++i) {
-        const int* e = pend + 8 * i;
-        if (!e[7]) continue;
-        // Head pairs: the unit's slots are consecutive, and when they fit in the idle K/V
-        // stages thread 0 brings them in with two bulk copies (one round trip instead of
-        // one per item batch) and every thread merges from shared memory. The (m, l) rows
-        // of a slot are 16-byte multiples only for an even slot_rows. (Measured slower in
-        // the fused llama8b step for 32-row units, so the one-head kernels keep the
-        // global merge.)
-        if constexpr (HP == 2) {
-          const uint32_t slot_bytes = static_cast<uint32_t>(p.slot_rows) * D * 4;
-          const uint32_t ml_bytes = static_cast<uint32_t>(p.slot_rows) * 8;
-          const int nsl = e[5];
-          if (p.slot_rows % 2 == 0 && static_cast<uint64_t>(nsl) * (slot_bytes + ml_bytes) <= C::RING_BYTES) {
-            float* so = reinterpret_cast<float*>(smem + C::OFF_K);
-            float2* sml = reinterpret_cast<float2*>(smem + C::OFF_K + nsl * slot_bytes);
-            if (threadIdx.x == 0) {
-              fence_async_global();  // the partials (generic stores) before the copy engine reads them
-              mbar_arrive_tx(merge_bar, nsl * (slot_bytes + ml_bytes));
-              bulk_load(smem_u32(so), p.partial_o + static_cast<int64_t>(e[4]) * p.slot_rows * D, nsl * slot_bytes,
-                        merge_bar);
-              bulk_load(smem_u32(sml), p.partial_ml + static_cast<int64_t>(e[4]) * p.slot_rows, nsl * ml_bytes,
-                        merge_bar);
-            }
-            const bool landed = mbar_wait(merge_bar, mphase & 1, abort_flag, p.status);
-            ++mphase;
-            if (landed) {
-              merge_staged<D>(p, e[0], 2 * e[1], e[2], e[3], so, sml, nsl, 0, threadIdx.x, C::THREADS);
-              merge_staged<D>(p, e[0], 2 * e[1] + 1, e[2], e[3], so, sml, nsl, p.rows, threadIdx.x, C::THREADS);
-            }
-            __syncthreads();  // the staging area is free for the next unit
-            continue;
-          }
-        }
-        // units of 128+ rows (a head pair, two M tiles) keep four items per thread in flight
-        constexpr int kItems = (HP == 2 || MT == 2) ? 4 : 1;
-        if (HP == 2) {  // the pair's heads, the second's rows after the first's in a slot
-          merge_unit<D, kItems>(p, e[0], 2 * e[1], e[2], e[3], e[4], e[5], threadIdx.x, C::THREADS, 0);
-          merge_unit<D, kItems>(p, e[0], 2 * e[1] + 1, e[2], e[3], e[4], e[5], threadIdx.x, C::THREADS,
-                                p.rows);
-        } else {
-          merge_unit<D, kItems>(p, e[0], e[1], e[2], e[3], e[4], e[5], threadIdx.x, C::THREADS);
-        }
-      }
-    }
   }
 }
 
@@ -895,6 +784,7 @@ cudaError_t launch_typed(const spec_attn_args_t& a, const AttnPlan& P, char* ws,
   // move real tiles away from blocks that pay no boundary.
   const int64_t units = static_cast<int64_t>(a.batch) * p.hunits * P.row_tiles;
   p.unit_overhead = units > P.grid ? Cf::UNIT_OVERHEAD : 0;
+  p.unit_heads = HP;
   if (!p.q_tma) mq = mk;  // unused
   const size_t smem = Cf::smem_bytes(a.batch);
   auto kernel = a.tree_mask ? attn_tc_kernel<D, MT, true, QR, HP> : attn_tc_kernel<D, MT, false, QR, HP>;
@@ -902,7 +792,8 @@ cudaError_t launch_typed(const spec_attn_args_t& a, const AttnPlan& P, char* ws,
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   kernel<<<P.grid, Cf::THREADS, smem, stream>>>(mk, mv, mq, p);
-  return cudaGetLastError();
+  e = cudaGetLastError();
+  return e != cudaSuccess ? e : launch_merge<D>(p, stream);
 }
 
 }  // namespace

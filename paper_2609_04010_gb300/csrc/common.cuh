@@ -135,6 +135,15 @@ cudaError_t launch_tree_build(const spec_tree_build_args_t& t, const TreeBuildLa
                               cudaStream_t stream, bool vec);
 
 // --- attention ---
+// A unit that was split between blocks, as the block that begins inside it leaves it to the
+// merge kernel.
+struct alignas(16) SplitUnit {
+  int b, g, rt;    // the unit: sequence, KV head (or group of heads), row tile
+  int slot0, nsl;  // its partial slots; nsl = 0: the block begins at a unit's start
+  int k;           // the block's left boundary is the unit's k-th
+  int pad[2];
+};
+
 struct AttnPlan {
   int path;          // SPEC_ATTN_CUDA_CORES or SPEC_ATTN_TENSOR_CORES
   int keys_on_lanes; // tensor cores: the keys-on-lanes kernel (attn_kl.cu), else row tiles
@@ -150,7 +159,7 @@ struct AttnPlan {
   int grid;          // blocks launched
   int slot_rows;     // rows per partial slot
   int64_t slots;     // partial slots
-  size_t tickets, partial_o, partial_ml, end;
+  size_t tickets, splits, partial_o, partial_ml, end;
 };
 
 AttnPlan attn_plan(const spec_attn_args_t& a, size_t base, int num_sms, int path_override);
