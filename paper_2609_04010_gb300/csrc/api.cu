@@ -36,6 +36,8 @@ int device_sm_count(int dev) {
 // each KV tile once per 16-row tile and issues the dot products on the FMA pipes), so
 // AUTO takes it whenever its shape limits allow.
 constexpr int kTcMinRows = 1;
+constexpr int kAcceptSms = 8;    // SMs a short attention leaves to a step's acceptance
+constexpr int kShortTiles = 64;  // 32 KB tiles per SM of a short attention
 int tc_min_rows() { return kTcMinRows; }
 
 namespace {
@@ -284,7 +286,17 @@ AttnPlan attn_plan(const spec_attn_args_t& a, size_t base, int num_sms, int path
     units = static_cast<int64_t>(a.batch) * (a.num_kv_heads / P.heads);
     P.nsplit = 1;
     P.tiles_per_split = 0;
-    P.grid = num_sms;
+    // In a step the acceptance's decisions and draws (short kernels of many small blocks) come
+    // when the attention blocks take the SMs, and a persistent block that finds its SM held
+    // by them starts late and delays the whole step. Where the attention is short enough to
+    // be delayed noticeably (at most kShortTiles 32 KB tiles per SM, about 50 us) it leaves
+    // them kAcceptSms: a step of 8 requests of 8 positions over 4,096 keys takes 55.4 us on
+    // every SM, 51.3 with 4 left, 47.3 with 8, 50.2 with 16; that attention alone 38.1 and
+    // 34.9. Longer ones use every SM (32 requests over up to 16,384 keys: 192.8 us against
+    // 195.5). Alone or in a step, a call's ranges are the same.
+    const int64_t tiles = units * ((static_cast<int64_t>(P.max_keys) * P.heads * a.head_dim * 2 + 16383) / 16384);
+    P.grid = tiles <= static_cast<int64_t>(kShortTiles) * num_sms && num_sms >= 16 * kAcceptSms
+                 ? num_sms - kAcceptSms : num_sms;
     P.slot_rows = P.heads * P.rows;
     P.slots = units + P.grid;
   } else if (P.keys_on_lanes) {

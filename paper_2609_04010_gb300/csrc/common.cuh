@@ -275,6 +275,24 @@ __device__ __forceinline__ float ex2(float x) {
   return y;
 }
 
+// The 16-byte granule at `a` (16-byte aligned) of a tensor that occupies [lo, hi), whose
+// first and last granules may hold bytes of others: those are read element by element
+// (E bytes each), bytes outside as zeros.
+template <int E>
+__device__ __forceinline__ uint4 load_granule(const char* a, const char* lo, const char* hi) {
+  if (a >= lo && a + 16 <= hi) return __ldg(reinterpret_cast<const uint4*>(a));
+  uint32_t w[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+  for (int i = 0; i < 16 / E; ++i) {
+    const char* x = a + i * E;
+    if (x >= lo && x + E <= hi) {
+      if (E == 4) w[i] = __ldg(reinterpret_cast<const uint32_t*>(x));
+      else w[i / 2] |= static_cast<uint32_t>(__ldg(reinterpret_cast<const uint16_t*>(x))) << (16 * (i & 1));
+    }
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
 // Programmatic dependent launch: let the next kernel on the stream start now / wait for
 // the kernel this one depends on (no-ops for kernels launched without the attribute).
 __device__ __forceinline__ void pdl_launch_dependents() {

@@ -249,3 +249,22 @@ def test_gpu_mean_accepted_matches_closed_form():
         se_k = np.sqrt(tail[k - 1] * (1 - tail[k - 1]) / N)
         assert abs(f - tail[k - 1]) < 5 * se_k + 1e-12, (k, f, tail[k - 1])
     print(f"mean accepted {a.mean():.4f} vs closed form {expect:.4f} (se {se:.4f})")
+
+
+@pytest.mark.parametrize("dtype,vocab", [("bf16", 4099), ("bf16", 4096), ("bf16", 33), ("bf16", 20001),
+                                         ("f32", 4097), ("f32", 2049), ("f32", 31), ("f32", 12290)])
+@pytest.mark.parametrize("shift", [0, 1, 3, 6])
+def test_rows_at_every_alignment(oracle_mod, dtype, vocab, shift):
+    # rows that start at every offset of a 16-byte granule: odd vocabularies, and tensors that
+    # begin `shift` elements into an allocation whose neighbours are NaN
+    inp = W.make_accept_inputs(5, 4, vocab, dtype, 3.0, 0.5, [1.0, 0.0, 0.7], seed=vocab + shift)
+    t = list(accept_tensors(inp))
+    for i in (0, 1):
+        flat = torch.full((t[i].numel() + 16,), float("nan"), dtype=t[i].dtype, device="cuda")
+        flat[shift:shift + t[i].numel()] = t[i].flatten()
+        t[i] = flat[shift:shift + t[i].numel()].view(t[i].shape)
+    r = binding.accept_block(*t)
+    torch.cuda.synchronize()
+    o = oracle_accept(oracle_mod, inp)
+    ties = compare_accept({k: v.cpu().numpy() for k, v in r.items()}, o, inp.gamma)
+    assert len(ties) <= 1, ties
