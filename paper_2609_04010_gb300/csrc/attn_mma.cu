@@ -104,9 +104,10 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
 template <int D, int HB, int MTW>
 __global__ void __launch_bounds__(MmaCfg<D, HB, MTW>::THREADS, 1)
     attn_mma_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ CUtensorMap tmap_v,
-                    AttnParams p, int box_keys) {
+                    AttnParams p, int page_shift, int box_shift) {
   using C = MmaCfg<D, HB, MTW>;
   constexpr int KS = C::KS, NS = C::NS, S = C::STAGES;
+  const int box_keys = 1 << box_shift;  // keys per copy (page and box sizes are powers of two)
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -144,8 +145,8 @@ __global__ void __launch_bounds__(MmaCfg<D, HB, MTW>::THREADS, 1)
   const int64_t total = pb[p.batch];
   const int ctas = range_count(total, p);
   const int cta = blockIdx.x;
-  const int64_t t0 = cta < ctas ? static_cast<int64_t>(cta) * total / ctas : 0;
-  const int64_t t1 = cta < ctas ? static_cast<int64_t>(cta + 1) * total / ctas : 0;
+  int64_t t0, t1;
+  block_range(p, pb, cta, total, ctas, t0, t1);
   const int OVH = p.unit_overhead;
 
   if (warp < 2) {
@@ -174,13 +175,13 @@ __global__ void __launch_bounds__(MmaCfg<D, HB, MTW>::THREADS, 1)
         if (!ok) break;
         const int key0 = (s.tile0 + k) * KS;
         // boxes with a visible key; a malformed sequence reads nothing
-        const int nbox = s.len_ok ? min(KS / box_keys, (s.kv_len - key0 + box_keys - 1) / box_keys) : 0;
+        const int nbox = s.len_ok ? min(KS >> box_shift, (s.kv_len - key0 + box_keys - 1) >> box_shift) : 0;
         bool bad = !s.len_ok;
         int page[KS / 16];
 #pragma unroll
         for (int q = 0; q < KS / 16; ++q)
           if (q < nbox) {
-            const int raw = page_of(s.b, (key0 + q * box_keys) / p.page_size);
+            const int raw = page_of(s.b, (key0 + (q << box_shift)) >> page_shift);
             const bool in_range = raw >= 0 && raw < p.num_pages;
             bad |= !in_range;
             page[q] = in_range ? raw : 0;  // an out-of-range page is read as page 0
@@ -192,7 +193,7 @@ __global__ void __launch_bounds__(MmaCfg<D, HB, MTW>::THREADS, 1)
 #pragma unroll
           for (int q = 0; q < KS / 16; ++q)
             if (q < nbox)
-              tma_load_group(ring + st * C::KV_BYTES + q * box_bytes, map, (key0 + q * box_keys) % p.page_size,
+              tma_load_group(ring + st * C::KV_BYTES + q * box_bytes, map, (key0 + (q << box_shift)) & (p.page_size - 1),
                              page[q] * p.hkv + s.g * HB, full(st));
         }
         __syncwarp();
@@ -266,8 +267,8 @@ __global__ void __launch_bounds__(MmaCfg<D, HB, MTW>::THREADS, 1)
         const uint32_t kst = sbase + st * C::KV_BYTES + head_off, vst = kst + C::OFF_V;
         auto step_off = [&](int n) {  // 16-key step n of the stage
           const int key = n * 16;
-          return static_cast<uint32_t>(key / box_keys) * (static_cast<uint32_t>(box_keys) * D * 2 * HB) +
-                 static_cast<uint32_t>(key % box_keys) * 128u;
+          return static_cast<uint32_t>(key >> box_shift) * (static_cast<uint32_t>(box_keys) * D * 2 * HB) +
+                 static_cast<uint32_t>(key & (box_keys - 1)) * 128u;
         };
         // ---- scores ----
         float sc[NS][2][4];
@@ -527,6 +528,12 @@ bool encode_group_map(CUtensorMap* map, const void* base, const spec_attn_args_t
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+int shift_of(int x) {
+  int s = 0;
+  while ((1 << s) < x) ++s;
+  return s;
+}
+
 template <int D, int HB, int MTW>
 cudaError_t launch_typed(const spec_attn_args_t& a, const AttnPlan& P, char* ws, cudaStream_t stream) {
   using C = MmaCfg<D, HB, MTW>;
@@ -542,12 +549,13 @@ cudaError_t launch_typed(const spec_attn_args_t& a, const AttnPlan& P, char* ws,
   p.grid = P.grid;
   p.min_tiles = kMmaMinTiles;
   p.unit_heads = HB;
+  p.whole_units = p.max_keys <= kWholeTiles * C::KS ? 1 : 0;
   const size_t smem = C::smem_bytes(a.batch);
   auto kernel = attn_mma_kernel<D, HB, MTW>;
   const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  kernel<<<P.grid, C::THREADS, smem, stream>>>(mk, mv, p, box_keys);
+  kernel<<<P.grid, C::THREADS, smem, stream>>>(mk, mv, p, shift_of(a.page_size), shift_of(box_keys));
   const cudaError_t launched = cudaGetLastError();
   return launched != cudaSuccess ? launched : launch_merge<D>(p, stream);
 }

@@ -263,8 +263,8 @@ __global__ void __launch_bounds__(TcCfg<D, MT, QR, HP>::THREADS, 1)
   const int64_t total = pb[p.batch];
   const int ctas = range_count(total, p);
   const int cta = blockIdx.x;
-  const int64_t t0 = cta < ctas ? static_cast<int64_t>(cta) * total / ctas : 0;
-  const int64_t t1 = cta < ctas ? static_cast<int64_t>(cta + 1) * total / ctas : 0;
+  int64_t t0, t1;
+  block_range(p, pb, cta, total, ctas, t0, t1);
   const int OVH = p.unit_overhead;
 
   if (pw >= 0) {
@@ -785,6 +785,7 @@ cudaError_t launch_typed(const spec_attn_args_t& a, const AttnPlan& P, char* ws,
   const int64_t units = static_cast<int64_t>(a.batch) * p.hunits * P.row_tiles;
   p.unit_overhead = units > P.grid ? Cf::UNIT_OVERHEAD : 0;
   p.unit_heads = HP;
+  p.whole_units = p.max_keys <= kWholeTiles * TK ? 1 : 0;
   if (!p.q_tma) mq = mk;  // unused
   const size_t smem = Cf::smem_bytes(a.batch);
   auto kernel = a.tree_mask ? attn_tc_kernel<D, MT, true, QR, HP> : attn_tc_kernel<D, MT, false, QR, HP>;
