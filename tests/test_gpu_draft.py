@@ -201,3 +201,21 @@ def test_commit_worked_examples_on_gpu(oracle_mod):
             np.testing.assert_array_equal(d_flags.cpu().numpy(), fl)
             assert int(d_count.cpu().numpy()[0]) == c
             np.testing.assert_array_equal(d_free.cpu().numpy()[:c], f[:c])
+
+
+@pytest.mark.parametrize("dtype,vocab", [("bf16", 4099), ("bf16", 33), ("bf16", 20001), ("bf16", 8 * 515),
+                                         ("f32", 4097), ("f32", 2049), ("f32", 31), ("f32", 4 * 1030)])
+@pytest.mark.parametrize("shift", [0, 1, 3])
+def test_sample_rows_at_every_alignment(oracle_mod, dtype, vocab, shift):
+    # odd vocabularies and tensors that begin inside a 16-byte granule, whose neighbours are NaN
+    dl, T, u = draft_inputs(5, 4, vocab, dtype, [1.0, 0.0, 0.7], seed=vocab + shift)
+    t = logits_dev(dl)
+    flat = torch.full((t.numel() + 16,), float("nan"), dtype=t.dtype, device="cuda")
+    flat[shift:shift + t.numel()] = t.flatten()
+    r = binding.sample_block(flat[shift:shift + t.numel()].view(t.shape), dev(T), dev(u))
+    torch.cuda.synchronize()
+    o = oracle_mod.sample_block(dl, T, u)
+    g, q = r["block_tokens"].cpu().numpy(), r["q_tok"].cpu().numpy()
+    same = g == o["tokens"]
+    assert np.all(same | (o["margin"] < TIE_MARGIN))
+    np.testing.assert_allclose(q[same], o["q_tok"][same], rtol=DIAG_RTOL)
