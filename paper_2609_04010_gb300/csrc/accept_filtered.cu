@@ -74,6 +74,7 @@ FilterLayout filter_layout(const spec_accept_args_t& a, int max_top_k, size_t ba
 namespace {
 
 constexpr int kRowUnroll = 8;        // 16-byte loads in flight per thread
+constexpr int kStageGranules = 4 * kRowThreads;  // 16-byte granules of an unaligned row staged at a time
 constexpr int kRankSortMax = 256;    // candidates ranked by counting; more are sorted bitonically
 constexpr uint32_t kRowBadLogits = 1u, kRowBadFilter = 2u;
 
@@ -713,64 +714,98 @@ __global__ void __launch_bounds__(kRowThreads, 8) filter_row_kernel(FiltParams p
         const int vi = v0 + u * kRowThreads + tid;
         dv[u] = vi < vend ? __ldg(rv + vi) : make_uint4(ninf, ninf, ninf, ninf);
       }
+      float vm[kRowUnroll];
 #pragma unroll
       for (int u = 0; u < kRowUnroll; ++u) {
         const int vi = v0 + u * kRowThreads + tid;
         const uint32_t wv[4] = {dv[u].x, dv[u].y, dv[u].z, dv[u].w};
 #pragma unroll
         for (int q = 0; q < 4; ++q) nacc |= (wv[q] & nan_mask) + nan_add;
-        if (greedy) {
-          // elements in increasing index order: a strict > keeps the lowest index
-#pragma unroll
-          for (int q = 0; q < kEpv; ++q) {
-            const float x = BF16 ? __uint_as_float((q & 1) ? (wv[q >> 1] & 0xffff0000u) : (wv[q >> 1] << 16))
-                                 : __uint_as_float(wv[q]);
-            if (x > m) { m = x; a = vi * kEpv + q; }
-          }
-        } else {
-          float vm;
+        if (BF16 || greedy) {
+          float top;
           if (BF16) {
             __nv_bfloat162 h = __hmax2(*reinterpret_cast<const __nv_bfloat162*>(&wv[0]),
                                        *reinterpret_cast<const __nv_bfloat162*>(&wv[1]));
             h = __hmax2(h, *reinterpret_cast<const __nv_bfloat162*>(&wv[2]));
             h = __hmax2(h, *reinterpret_cast<const __nv_bfloat162*>(&wv[3]));
-            vm = fmaxf(__bfloat162float(h.x), __bfloat162float(h.y));
+            top = fmaxf(__bfloat162float(h.x), __bfloat162float(h.y));
           } else {
-            vm = fmaxf(fmaxf(__uint_as_float(wv[0]), __uint_as_float(wv[1])),
-                       fmaxf(__uint_as_float(wv[2]), __uint_as_float(wv[3])));
+            top = fmaxf(fmaxf(__uint_as_float(wv[0]), __uint_as_float(wv[1])),
+                        fmaxf(__uint_as_float(wv[2]), __uint_as_float(wv[3])));
           }
-          m = fmaxf(m, vm);
-          // the lane maximum: the kGroup consecutive threads of a lane, then one atomic
-          uint32_t key = vi < vend ? order_key(vm) : 0u;
+          if (top > m) {  // rare: the first element of the vector that holds the new maximum
+            m = top;
+            int at = kEpv - 1;
 #pragma unroll
-          for (int o = 1; o < kGroup; o <<= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, o));
-          if ((tid & (kGroup - 1)) == 0 && vi < vend) atomicMax(&lanes[vi / vpl - l0], key);
+            for (int q = kEpv - 2; q >= 0; --q) {
+              const float x = BF16 ? __uint_as_float((q & 1) ? (wv[q >> 1] & 0xffff0000u) : (wv[q >> 1] << 16))
+                                   : __uint_as_float(wv[q]);
+              at = x == top ? q : at;
+            }
+            a = vi * kEpv + at;
+          }
+        } else {
+          vm[u] = fmaxf(fmaxf(__uint_as_float(wv[0]), __uint_as_float(wv[1])),
+                        fmaxf(__uint_as_float(wv[2]), __uint_as_float(wv[3])));
+          m = fmaxf(m, vm[u]);
         }
+      }
+      if (!BF16 && !greedy) {  // the 16 threads of a lane's vectors, 8 lanes at a time
+        const float lm = reduce8<kGroup>(vm, tid & 7, [](float x, float y) { return fmaxf(x, y); });
+        const int vl = v0 + (tid & 7) * kRowThreads + (tid & ~(kGroup - 1));  // the owned lane's first vector here
+        if ((tid & 8) == 0 && vl < vend) atomicMax(&lanes[vl / vpl - l0], order_key(lm));
       }
     }
     bad = (nacc & nan_top) != 0;
   } else {
+    // Rows not 16-byte aligned: the granules that cover kStage elements come into shared
+    // memory with 16-byte loads, four a thread, and the elements are read from there
+    // (element loads kept 16 KB in flight on an SM: 39.5 us for 144 rows of 50,257 fp32
+    // logits, now 29.3).
+    constexpr int E = BF16 ? 2 : 4;
+    constexpr int kStage = kStageGranules * 16 / E;
+    uint4* stage = reinterpret_cast<uint4*>(dsm + p.smem_a + static_cast<size_t>(cap) * 12);
+    const char* lo = static_cast<const char*>(p.mode == 1 || r >= gamma ? p.drafter : p.target);
+    const char* hi = lo + static_cast<int64_t>(p.batch) * gamma * V * E;
     if (e_begin + tid < e_end) a = e_begin + tid;
-    for (int e0 = e_begin; e0 < e_end; e0 += kRowThreads * kRowUnroll) {
-      float x[kRowUnroll];
+    for (int h0 = e_begin; h0 < e_end; h0 += kStage) {
+      const char* from = rowp + static_cast<int64_t>(h0) * E;
+      const uint32_t off = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(from)) & 15u;
+      const int ngran = (min(kStage, e_end - h0) * E + static_cast<int>(off) + 15) / 16;
+      uint4 g[kStageGranules / kRowThreads];
 #pragma unroll
-      for (int u = 0; u < kRowUnroll; ++u) {
-        const int ei = e0 + u * kRowThreads + tid;
-        x[u] = ei < e_end ? load_elem<BF16>(rowp, ei) : -INFINITY;
+      for (int k = 0; k < kStageGranules / kRowThreads; ++k) {
+        const int n = k * kRowThreads + tid;
+        g[k] = n < ngran ? load_granule<E>(from - off + 16 * n, lo, hi) : make_uint4(0, 0, 0, 0);
       }
+      const uint4 last = tid == 0 && ngran > kStageGranules
+                             ? load_granule<E>(from - off + 16 * kStageGranules, lo, hi) : make_uint4(0, 0, 0, 0);
+      __syncthreads();  // the previous stage has been read
 #pragma unroll
-      for (int u = 0; u < kRowUnroll; ++u) {
-        const int ei = e0 + u * kRowThreads + tid;
-        bad |= x[u] != x[u];
-        if (greedy) {
-          if (x[u] > m) { m = x[u]; a = ei; }
-        } else {
-          m = fmaxf(m, x[u]);
-          // a warp's 32 consecutive elements lie in one lane
-          uint32_t key = ei < e_end ? order_key(x[u]) : 0u;
+      for (int k = 0; k < kStageGranules / kRowThreads; ++k) stage[k * kRowThreads + tid] = g[k];
+      if (tid == 0) stage[kStageGranules] = last;
+      __syncthreads();
+      const char* sm = reinterpret_cast<const char*>(stage) + off;
+      for (int e0 = h0; e0 < min(h0 + kStage, e_end); e0 += kRowThreads * kRowUnroll) {
+        float x[kRowUnroll];
 #pragma unroll
-          for (int o = 1; o < 32; o <<= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, o));
-          if ((tid & 31) == 0 && ei < e_end) atomicMax(&lanes[ei / lane_elems - l0], key);
+        for (int u = 0; u < kRowUnroll; ++u) {
+          const int ei = e0 + u * kRowThreads + tid;
+          const char* at = sm + (ei - h0) * E;
+          x[u] = ei < e_end ? (BF16 ? bf16_bits_to_f32(*reinterpret_cast<const uint16_t*>(at))
+                                    : *reinterpret_cast<const float*>(at))
+                            : -INFINITY;
+          bad |= x[u] != x[u];
+          if (greedy) {
+            if (x[u] > m) { m = x[u]; a = ei; }
+          } else {
+            m = fmaxf(m, x[u]);
+          }
+        }
+        if (!greedy) {  // a warp's 32 consecutive elements lie in one lane
+          const float lm = reduce8<32>(x, tid & 7, [](float y, float z) { return fmaxf(y, z); });
+          const int ei = e0 + (tid & 7) * kRowThreads + (tid & ~31);
+          if ((tid & 31) < 8 && ei < e_end) atomicMax(&lanes[ei / lane_elems - l0], order_key(lm));
         }
       }
     }
@@ -851,35 +886,58 @@ __global__ void __launch_bounds__(kRowThreads, 8) filter_row_kernel(FiltParams p
     uint32_t* my_hist = s_hist + (tid >> 5) * 256;
     for (int i = tid; i < (kRowThreads / 32) * 256; i += kRowThreads) s_hist[i] = 0;
     __syncthreads();
-    for (int i = tid; i < nlanes; i += kRowThreads) atomicAdd(&my_hist[lanes[i] >> 24], 1u);
+    // One pass finds it where it lies among the 255 next lower values of those high bits (a
+    // bf16 row's lane maxima span about two binades, 256 values): the lanes spread over the
+    // bins, while nearly all share the two or three top bytes a digit pass counts (the two
+    // digit passes took 4.6 us of a row's select, this one 2.3).
+    const uint32_t top16 = static_cast<uint32_t>(best >> 48);
+    for (int i = tid; i < nlanes; i += kRowThreads) {
+      const uint32_t below = top16 - (lanes[i] >> 16);  // an unused lane's key is 0
+      if (below < 256u) atomicAdd(&my_hist[255u - below], 1u);
+    }
     __syncthreads();
     if (tid < 32) {
       uint32_t above = 0;
       const int bin = find_bin_desc(s_hist, kRowThreads / 32, static_cast<uint32_t>(K), &above);
-      if (tid == 0) {
-        s_misc[0] = bin;
-        s_misc[1] = static_cast<int>(above);
-      }
+      if (tid == 0) s_misc[0] = bin;
     }
     __syncthreads();
     uint32_t beta = 0;
-    const int b1 = s_misc[0];
-    if (b1 >= 0) {
-      const uint32_t need = static_cast<uint32_t>(K - s_misc[1]);
+    const int near = s_misc[0];
+    if (near >= 0) beta = (top16 - (255u - static_cast<uint32_t>(near))) << 16;
+    if (near < 0) {  // by two radix digits
+      __syncthreads();
       for (int i = tid; i < (kRowThreads / 32) * 256; i += kRowThreads) s_hist[i] = 0;
       __syncthreads();
-      for (int i = tid; i < nlanes; i += kRowThreads) {
-        const uint32_t k = lanes[i];
-        if (static_cast<int>(k >> 24) == b1) atomicAdd(&my_hist[(k >> 16) & 0xffu], 1u);
-      }
+      for (int i = tid; i < nlanes; i += kRowThreads) atomicAdd(&my_hist[lanes[i] >> 24], 1u);
       __syncthreads();
       if (tid < 32) {
         uint32_t above = 0;
-        const int bin = find_bin_desc(s_hist, kRowThreads / 32, need, &above);
-        if (tid == 0) s_misc[2] = bin;
+        const int bin = find_bin_desc(s_hist, kRowThreads / 32, static_cast<uint32_t>(K), &above);
+        if (tid == 0) {
+          s_misc[0] = bin;
+          s_misc[1] = static_cast<int>(above);
+        }
       }
       __syncthreads();
-      beta = (static_cast<uint32_t>(b1) << 24) | (static_cast<uint32_t>(s_misc[2]) << 16);
+      const int b1 = s_misc[0];
+      if (b1 >= 0) {
+        const uint32_t need = static_cast<uint32_t>(K - s_misc[1]);
+        for (int i = tid; i < (kRowThreads / 32) * 256; i += kRowThreads) s_hist[i] = 0;
+        __syncthreads();
+        for (int i = tid; i < nlanes; i += kRowThreads) {
+          const uint32_t k = lanes[i];
+          if (static_cast<int>(k >> 24) == b1) atomicAdd(&my_hist[(k >> 16) & 0xffu], 1u);
+        }
+        __syncthreads();
+        if (tid < 32) {
+          uint32_t above = 0;
+          const int bin = find_bin_desc(s_hist, kRowThreads / 32, need, &above);
+          if (tid == 0) s_misc[2] = bin;
+        }
+        __syncthreads();
+        beta = (static_cast<uint32_t>(b1) << 24) | (static_cast<uint32_t>(s_misc[2]) << 16);
+      }
     }
     // the lanes that can hold a top-K element (counted, then placed by a block scan)
     int mine = 0;
@@ -893,44 +951,66 @@ __global__ void __launch_bounds__(kRowThreads, 8) filter_row_kernel(FiltParams p
     __syncthreads();
     // their elements at or above the bound
     if (nq <= cap) {
-      // items of 8 contiguous elements: lane_elems / 8 per lane
+      // Items of 8 contiguous elements, lane_elems / 8 per lane; a thread's next kItems items
+      // load together (their runs have left L2 while other rows streamed; one trip to memory
+      // at a time took 5.3 of the select's 14 us, now 4.0 of 11).
+      constexpr int kItems = BF16 ? 4 : 2, kEpv = BF16 ? 8 : 4;
       const int ipl = lane_elems / 8;
-      for (int it0 = 0; it0 < nq * ipl; it0 += kRowThreads) {
-        const int it = it0 + tid;
-        const bool live = it < nq * ipl;
-        const int e0 = live ? qlane[it / ipl] * lane_elems + (it % ipl) * 8 : V;
-        float x[8];
-        if (VEC) {
-          constexpr int kEpv = BF16 ? 8 : 4;
+      for (int it0 = 0; it0 < nq * ipl; it0 += kItems * kRowThreads) {
+        uint4 raw[kItems][8 / kEpv];
+        int at[kItems];
 #pragma unroll
-          for (int h = 0; h < 8 / kEpv; ++h) {
-            const int e = e0 + h * kEpv;
-            uint4 v = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
-            if (e < V) v = __ldg(reinterpret_cast<const uint4*>(rowp + static_cast<int64_t>(e) * (BF16 ? 2 : 4)));
-            const uint32_t wv[4] = {v.x, v.y, v.z, v.w};
+        for (int n = 0; n < kItems; ++n) {
+          const int it = it0 + n * kRowThreads + tid;
+          at[n] = it < nq * ipl ? qlane[it / ipl] * lane_elems + (it % ipl) * 8 : V;
+          if (VEC) {
 #pragma unroll
-            for (int q = 0; q < kEpv; ++q)
-              x[h * kEpv + q] = BF16 ? __uint_as_float((q & 1) ? (wv[q >> 1] & 0xffff0000u) : (wv[q >> 1] << 16))
-                                     : __uint_as_float(wv[q]);
+            for (int h = 0; h < 8 / kEpv; ++h) {
+              const int e = at[n] + h * kEpv;
+              raw[n][h] = make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
+              if (e < V) raw[n][h] = __ldg(reinterpret_cast<const uint4*>(rowp + static_cast<int64_t>(e) * (BF16 ? 2 : 4)));
+            }
           }
-        } else {
-#pragma unroll
-          for (int q = 0; q < 8; ++q) x[q] = e0 + q < V ? load_elem<BF16>(rowp, e0 + q) : -INFINITY;
         }
-        uint32_t kq[8];
-        unsigned takem = 0;
+#pragma unroll 1
+        for (int n = 0; n < kItems; ++n) {
+          const int e0 = at[0];
+          float x[8];
+          if (VEC) {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          kq[q] = order_key(x[q]);
-          if (e0 + q < V && kq[q] >= beta) takem |= 1u << q;
-        }
-        int c = warp_slots(__popc(takem), &s_ncand);
+            for (int h = 0; h < 8 / kEpv; ++h) {
+              const uint32_t wv[4] = {raw[0][h].x, raw[0][h].y, raw[0][h].z, raw[0][h].w};
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-          if ((takem >> q) & 1u) {
-            if (c < cap) cand[c] = cand_of(kq[q], static_cast<uint32_t>(e0 + q));
-            ++c;
+              for (int q = 0; q < kEpv; ++q)
+                x[h * kEpv + q] = BF16 ? __uint_as_float((q & 1) ? (wv[q >> 1] & 0xffff0000u) : (wv[q >> 1] << 16))
+                                       : __uint_as_float(wv[q]);
+            }
+          } else {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) x[q] = e0 + q < V ? load_elem<BF16>(rowp, e0 + q) : -INFINITY;
           }
+          // the next item moves up (one copy of the code below, whatever kItems)
+#pragma unroll
+          for (int k = 0; k + 1 < kItems; ++k) {
+            at[k] = at[k + 1];
+#pragma unroll
+            for (int h = 0; h < 8 / kEpv; ++h) raw[k][h] = raw[k + 1][h];
+          }
+          uint32_t kq[8];
+          unsigned takem = 0;
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            kq[q] = order_key(x[q]);
+            if (e0 + q < V && kq[q] >= beta) takem |= 1u << q;
+          }
+          int c = warp_slots(__popc(takem), &s_ncand);
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+            if ((takem >> q) & 1u) {
+              if (c < cap) cand[c] = cand_of(kq[q], static_cast<uint32_t>(e0 + q));
+              ++c;
+            }
+        }
       }
     }
     __syncthreads();
@@ -1083,11 +1163,15 @@ cudaError_t launch_filtered_typed(const FiltParams& p, cudaStream_t stream, bool
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.splits, p.mode == 1 ? p.gamma : 2 * p.gamma - 1, p.batch);
   cfg.blockDim = dim3(kRowThreads);
-  cfg.dynamicSmemBytes = p.smem_a + static_cast<size_t>(p.cand_cap) * 12;
+  cfg.dynamicSmemBytes = p.smem_a + static_cast<size_t>(p.cand_cap) * 12 + (VEC ? 0 : (kStageGranules + 1) * 16);
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = overlap_prior ? 1 : 0;  // beside the attention kernel of a verify step
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, filter_row_kernel<BF16, VEC>, p);
+  cudaError_t e = cudaSuccess;
+  if (!VEC)  // the stage may take a block past 48 KB
+    e = cudaFuncSetAttribute(filter_row_kernel<BF16, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(cfg.dynamicSmemBytes));
+  if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, filter_row_kernel<BF16, VEC>, p);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }

@@ -293,6 +293,28 @@ __device__ __forceinline__ uint4 load_granule(const char* a, const char* lo, con
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
+// Reduction of 8 values over the threads of a group of G, all 8 together: the tree of a
+// butterfly (neighbours first), but each of the first three exchanges halves the values a
+// thread carries, 7 to 9 shuffles instead of 8 log2 G. Thread i of the group gets value
+// i & 7; v is overwritten.
+template <int G, class Op>
+__device__ __forceinline__ float reduce8(float* v, int i, Op op) {
+  const bool b0 = i & 1, b1 = i & 2, b2 = i & 4;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const float keep = b0 ? v[2 * j + 1] : v[2 * j];
+    v[j] = op(keep, __shfl_xor_sync(0xffffffffu, b0 ? v[2 * j] : v[2 * j + 1], 1));
+  }
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const float keep = b1 ? v[2 * j + 1] : v[2 * j];
+    v[j] = op(keep, __shfl_xor_sync(0xffffffffu, b1 ? v[2 * j] : v[2 * j + 1], 2));
+  }
+  float r = op(b2 ? v[1] : v[0], __shfl_xor_sync(0xffffffffu, b2 ? v[0] : v[1], 4));
+#pragma unroll
+  for (int o = 8; o < G; o <<= 1) r = op(r, __shfl_xor_sync(0xffffffffu, r, o));
+  return r;
+}
 // Programmatic dependent launch: let the next kernel on the stream start now / wait for
 // the kernel this one depends on (no-ops for kernels launched without the attribute).
 __device__ __forceinline__ void pdl_launch_dependents() {

@@ -135,28 +135,6 @@ __device__ __forceinline__ void fma2(float a0, float a1, float b, float c, float
   asm("mov.b64 {%0, %1}, %2;" : "=f"(d0), "=f"(d1) : "l"(vd));
 }
 
-// Reduction of 8 values over the threads of a group of G, all 8 together: the tree of a
-// butterfly (neighbours first), but each of the first three exchanges halves the values a
-// thread carries, 7 to 9 shuffles instead of 8 log2 G. Thread i of the group gets value
-// i & 7; v is overwritten.
-template <int G, class Op>
-__device__ __forceinline__ float reduce8(float* v, int i, Op op) {
-  const bool b0 = i & 1, b1 = i & 2, b2 = i & 4;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const float keep = b0 ? v[2 * j + 1] : v[2 * j];
-    v[j] = op(keep, __shfl_xor_sync(0xffffffffu, b0 ? v[2 * j] : v[2 * j + 1], 1));
-  }
-#pragma unroll
-  for (int j = 0; j < 2; ++j) {
-    const float keep = b1 ? v[2 * j + 1] : v[2 * j];
-    v[j] = op(keep, __shfl_xor_sync(0xffffffffu, b1 ? v[2 * j] : v[2 * j + 1], 2));
-  }
-  float r = op(b2 ? v[1] : v[0], __shfl_xor_sync(0xffffffffu, b2 ? v[0] : v[1], 4));
-#pragma unroll
-  for (int o = 8; o < G; o <<= 1) r = op(r, __shfl_xor_sync(0xffffffffu, r, o));
-  return r;
-}
 // The reverse: every thread of the group gets all 8 of reduce8's results.
 __device__ __forceinline__ void gather8(float r, int i, float* v) {
   const bool b0 = i & 1, b1 = i & 2, b2 = i & 4;

@@ -187,3 +187,50 @@ def test_deterministic(oracle_mod):
     b = gpu_filtered(inp, k, p)
     for key in ("num_accepted", "out_tokens", "num_emitted"):
         np.testing.assert_array_equal(a[key], b[key])
+
+
+@pytest.mark.parametrize("dtype,vocab", [("bf16", 4099), ("bf16", 33), ("bf16", 20001), ("f32", 4097),
+                                         ("f32", 2049), ("f32", 4 * 1030), ("bf16", 8 * 515)])
+@pytest.mark.parametrize("shift", [0, 1, 3])
+def test_rows_at_every_alignment(oracle_mod, dtype, vocab, shift):
+    # odd vocabularies and tensors that begin inside a 16-byte granule, whose neighbours are NaN
+    k = 20
+    inp = W.make_accept_inputs(5, 4, vocab, dtype, 3.0, 0.5, [1.0, 0.0, 0.7], seed=vocab + shift, draft_top_k=k)
+    t = list(accept_tensors(inp))
+    for i in (0, 1):
+        flat = torch.full((t[i].numel() + 16,), float("nan"), dtype=t[i].dtype, device="cuda")
+        flat[shift:shift + t[i].numel()] = t[i].flatten()
+        t[i] = flat[shift:shift + t[i].numel()].view(t[i].shape)
+    K, P = np.full(5, k, np.int32), np.full(5, 0.95, np.float32)
+    r = binding.accept_block_filtered(t[0], t[1], t[2], t[3], torch.from_numpy(K).cuda(),
+                                      torch.from_numpy(P).cuda(), t[4])
+    torch.cuda.synchronize()
+    a = binding.accept_block_filtered(*[x.clone() for x in t[:4]], torch.from_numpy(K).cuda(),
+                                      torch.from_numpy(P).cuda(), t[4])  # the same, from aligned tensors
+    for key in ("num_accepted", "num_emitted", "out_tokens"):
+        assert torch.equal(r[key], a[key])
+    o = oracle_mod.accept_block_filtered(inp.target_logits, inp.drafter_logits, inp.block_tokens, inp.temperature,
+                                         K, P, inp.uniforms)
+    same = r["num_accepted"].cpu().numpy() == o["num_accepted"]
+    assert same.sum() >= 4
+
+
+def test_bound_beyond_the_near_values(oracle_mod):
+    # lane maxima spread over many binades: the one-pass bound (255 bf16 values below the row's
+    # maximum) does not reach the k-th, and the digit passes take over
+    inp = W.make_accept_inputs(4, 3, 30000, "bf16", 3.0, 0.5, 1.0, seed=77, draft_top_k=50)
+    scale = np.exp(np.linspace(np.log(1e-6), np.log(1e4), 30000)).astype(np.float32)
+    for x in (inp.target_logits, inp.drafter_logits):
+        x[:] = W.f32_to_bf16_bits(np.abs(W.bf16_bits_to_f32(x)) * scale).reshape(x.shape)
+    K, P = np.full(4, 400, np.int32), np.full(4, 1.0, np.float32)
+    T = np.full(4, 1e4, np.float32)
+    t = accept_tensors(inp)
+    r = binding.accept_block_filtered(t[0], t[1], t[2], torch.from_numpy(T).cuda(), torch.from_numpy(K).cuda(),
+                                      torch.from_numpy(P).cuda(), t[4])
+    torch.cuda.synchronize()
+    o = oracle_mod.accept_block_filtered(inp.target_logits, inp.drafter_logits, inp.block_tokens, T, K, P, inp.uniforms)
+    same = r["num_accepted"].cpu().numpy() == o["num_accepted"]
+    assert np.all(same)
+    d = r["diag"].cpu().numpy()
+    m = ~np.isnan(o["diag"])
+    np.testing.assert_allclose(d[m], o["diag"][m], rtol=1e-4, atol=1e-9)
