@@ -43,11 +43,8 @@ TreeLayout tree_layout(int batch, int nodes, int vocab, size_t base, int sms, bo
   L.elems_per_split = static_cast<int>((nlanes + splits - 1) / splits) * lane;
   L.splits = (vocab + L.elems_per_split - 1) / L.elems_per_split;
   L.tickets = base;
-  L.row_tickets = ws_round(L.tickets + sizeof(uint32_t) * batch);
-  L.parts = ws_round(L.row_tickets + sizeof(uint32_t) * rows);
-  L.argmax = ws_round(L.parts + 16 * rows * L.splits);
-  L.rowstat = ws_round(L.argmax + sizeof(int32_t) * rows);
-  L.end = ws_round(L.rowstat + sizeof(float) * 2 * rows);
+  L.parts = ws_round(L.tickets + sizeof(uint32_t) * batch);
+  L.end = ws_round(L.parts + 16 * rows * L.splits);
   return L;
 }
 
@@ -67,10 +64,7 @@ struct TreeParams {
   int32_t* num_emitted;    // [batch]
   uint32_t* status;
   uint32_t* tickets;
-  uint32_t* row_tickets;
   uint4* parts;
-  int32_t* argmax;         // [batch][nodes]; -1 marks an unusable row
-  float2* rowstat;         // [batch][nodes]: (max logit, sum of 2^((l - max) log2e / T))
   const float* temperature;  // [batch] or NULL (greedy)
   const float* uniforms;     // [batch][nodes]
 };
@@ -100,7 +94,13 @@ __global__ void __launch_bounds__(kThreads, kTreeBlocksPerSm) tree_greedy_kernel
   __shared__ unsigned long long s_red[kThreads / 32];
   __shared__ float s_fsum[kThreads / 32];
   __shared__ int s_bad, s_last;
-  __shared__ int s_arg[64];
+  // the sequence's last block: its rows' argmax, (max, sum) and parts (max, sum), its nodes
+  __shared__ int s_arg[64], s_tok_in[64], s_par[64], s_acc[64];
+  __shared__ float2 s_stat[64], s_part[64 * 16];
+  __shared__ double s_e[64];
+  __shared__ uint32_t s_badin;
+  __shared__ int s_lo, s_hi;
+  __shared__ double s_excl;
   // hand-off from the walking warp to the sampled final draw
   __shared__ int s_final, s_len, s_nrm, s_kcross, s_tok;
   __shared__ int s_rm[64];                 // tokens rejected at the final node, ascending
@@ -208,266 +208,181 @@ __global__ void __launch_bounds__(kThreads, kTreeBlocksPerSm) tree_greedy_kernel
     for (int k = 0; k < kThreads / 32; ++k) part_sum += s_fsum[k];
   }
 
-  float2 stat = make_float2(key_to_float(static_cast<uint32_t>(best >> 32)), part_sum);
-  if (p.splits > 1 || tempered) {
-    if (tid == 0)
-      p.parts[rid * p.splits + split] = make_uint4(static_cast<uint32_t>(best), static_cast<uint32_t>(best >> 32),
-                                                   static_cast<uint32_t>(s_bad), __float_as_uint(part_sum));
-  }
-  if (p.splits > 1) {
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) {
-      const uint32_t prev = atomicAdd(&p.row_tickets[rid], 1u);
-      s_last = prev == static_cast<uint32_t>(p.splits - 1);
-      if (s_last) p.row_tickets[rid] = 0;
-    }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    if (tid < 32) {
-      unsigned long long bb = 0ull;
-      uint32_t anybad = 0;
-      for (int k = tid; k < p.splits; k += 32) {
-        const uint4 q = __ldcg(p.parts + rid * p.splits + k);
-        const unsigned long long c = (static_cast<unsigned long long>(q.y) << 32) | q.x;
-        bb = c > bb ? c : bb;
-        anybad |= q.z;
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long y = __shfl_xor_sync(0xffffffffu, bb, o);
-        bb = y > bb ? y : bb;
-      }
-      anybad = __reduce_or_sync(0xffffffffu, anybad);
-      // the row's sum relative to its maximum
-      const float M = key_to_float(static_cast<uint32_t>(bb >> 32));
-      float z = 0.f;
-      if (tempered && M > -INFINITY && M < INFINITY) {
-        for (int k = tid; k < p.splits; k += 32) {
-          const uint4 q = __ldcg(p.parts + rid * p.splits + k);
-          z += __uint_as_float(q.w) * rel_weight(key_to_float(q.y), M, cs);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-      }
-      if (tid == 0) {
-        s_red[0] = bb;
-        s_bad = anybad ? 1 : 0;
-        s_fsum[0] = z;
-      }
-    }
-    __syncthreads();
-    best = s_red[0];
-    stat = make_float2(key_to_float(static_cast<uint32_t>(best >> 32)), s_fsum[0]);
-  }
+  // The sequence's last block (one ticket for all parts of all its rows: a ticket per row
+  // and another per sequence were two fences and atomics in a row) has every row's parts.
   if (tid == 0) {
-    // a tempered row needs a finite maximum (NaN and +inf are flagged above)
-    const bool unusable = s_bad || (tempered && !(stat.x > -INFINITY));
-    p.argmax[rid] = unusable ? -1 : static_cast<int>(0xffffffffu - static_cast<uint32_t>(best));
-    if (tempered) p.rowstat[rid] = stat;
-  }
-
-  // the sequence's last row block walks the tree
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) {
+    p.parts[rid * p.splits + split] = make_uint4(static_cast<uint32_t>(best), static_cast<uint32_t>(best >> 32),
+                                                 static_cast<uint32_t>(s_bad), __float_as_uint(part_sum));
+    __threadfence();
     const uint32_t prev = atomicAdd(&p.tickets[b], 1u);
-    s_last = prev == static_cast<uint32_t>(N - 1);
-    if (s_last) p.tickets[b] = 0;
+    s_last = prev == static_cast<uint32_t>(N * p.splits - 1);
+    if (s_last) p.tickets[b] = 0;  // leave the counter at zero for the next call
+    s_final = -1;
+    s_badin = 0;
   }
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  if (tid < N) s_arg[tid] = __ldcg(p.argmax + static_cast<int64_t>(b) * N + tid);
-  if (tid == 0) s_final = -1;
-  __syncthreads();
   const int64_t brow = static_cast<int64_t>(b) * N;
-  int32_t* path = p.path + brow;
-  int32_t* out = p.out_tokens + static_cast<int64_t>(b) * (N + 1);
-  if (tid < 32) {
-    // one warp: lane c holds node c (N <= 64: two nodes per lane)
-    const int lane = tid;
-    int tok[2], par[2];
-    uint32_t bad_in = 0;
+  {
+    // 16 threads per row, a part each (at most kFiltMaxSplits = 16), 8 rows at a time; all
+    // loads in flight together
+    const int k = tid & 15, g = tid >> 4;
+    uint4 q[8];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int c = lane + 32 * h;
-      tok[h] = c < N ? p.tokens[brow + c] : -1;
-      par[h] = c < N ? p.parents[brow + c] : -2;
-      if (c < N) {
-        if (tok[h] < 0 || tok[h] >= V) bad_in |= SPEC_FLAG_BAD_TOKEN;
-        if (c == 0 ? par[h] != -1 : (par[h] < 0 || par[h] >= c)) bad_in |= SPEC_FLAG_BAD_TREE;
-        if (s_arg[c] < 0) bad_in |= SPEC_FLAG_BAD_LOGITS;
-      }
+    for (int i = 0; i < 8; ++i) {
+      const int row = g + 8 * i;
+      q[i] = row < N && k < p.splits ? __ldcg(p.parts + (brow + row) * p.splits + k) : make_uint4(0u, 0u, 0u, 0u);
     }
-    bad_in = __reduce_or_sync(0xffffffffu, bad_in);
-    if (bad_in) {
-      for (int c = lane; c < N; c += 32) path[c] = -1;
-      for (int c = lane; c <= N; c += 32) out[c] = -1;
-      if (lane == 0) {
-        p.num_accepted[b] = -1;
-        p.num_emitted[b] = 0;
-        set_status(p.status, bad_in);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int row = g + 8 * i;
+      if (8 * i >= N) break;
+      unsigned long long bb = (static_cast<unsigned long long>(q[i].y) << 32) | q[i].x;
+      uint32_t rbad = q[i].z;
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) {
+        const unsigned long long y = __shfl_xor_sync(0xffffffffu, bb, o);
+        bb = y > bb ? y : bb;
+        rbad |= __shfl_xor_sync(0xffffffffu, rbad, o);
       }
-    } else {
-      int cur = 0, len = 1;
-      if (lane == 0) {
-        path[0] = 0;
-        out[0] = tok[0];  // the root: lane 0 holds node 0
-      }
-      if (!tempered) {
-        for (int step = 1; step < N; ++step) {
-          const int want = s_arg[cur];
-          const unsigned m0 = __ballot_sync(0xffffffffu, par[0] == cur && tok[0] == want);
-          const unsigned m1 = __ballot_sync(0xffffffffu, par[1] == cur && tok[1] == want);
-          int nxt = -1;
-          if (m0) nxt = __ffs(m0) - 1;
-          else if (m1) nxt = 32 + __ffs(m1) - 1;
-          if (nxt < 0) break;
-          const int t = __shfl_sync(0xffffffffu, nxt < 32 ? tok[0] : tok[1], nxt & 31);
-          if (lane == 0) {
-            path[len] = nxt;
-            out[len] = t;
-          }
-          cur = nxt;
-          ++len;
+      const float M = key_to_float(static_cast<uint32_t>(bb >> 32)), pm = key_to_float(q[i].y);
+      const float pw = __uint_as_float(q[i].w);
+      // the row's sum relative to its maximum
+      float z = tempered && M > -INFINITY && M < INFINITY && k < p.splits ? pw * rel_weight(pm, M, cs) : 0.f;
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+      if (row < N) {
+        s_part[row * 16 + k] = make_float2(pm, pw);
+        if (k == 0) {
+          // a tempered row needs a finite maximum (NaN and +inf are flagged by its parts)
+          const bool unusable = rbad != 0 || (tempered && !(M > -INFINITY));
+          s_arg[row] = unusable ? -1 : static_cast<int>(0xffffffffu - static_cast<uint32_t>(bb));
+          s_stat[row] = make_float2(M, z);
         }
-        for (int c = len + lane; c < N; c += 32) path[c] = -1;
-        if (lane == 0) out[len] = s_arg[cur];
-        for (int c = len + 1 + lane; c <= N; c += 32) out[c] = -1;
-        if (lane == 0) {
-          p.num_accepted[b] = len - 1;
-          p.num_emitted[b] = len + 1;
-        }
-      } else {
-        // sampled walk: the children of the current node, in node order, are point-mass
-        // proposals; child c is accepted iff u[c] <= p'(token), p' the node's target
-        // distribution without the tokens of the siblings rejected before it.
-        // Everything a step reads is fixed by the tree, so it is gathered once, for all
-        // nodes at the same time: each node's weight e_c = exp((l(t_c) - M) / T) in fp64
-        // under its parent's row (M that row's maximum; 0 for a repeated sibling token,
-        // removed with its first occurrence), the weight of its earlier siblings in node
-        // order, its own row's (maximum, sum) and its uniform.
-        const char* tbase = static_cast<const char*>(p.target);
-        const size_t rbytes = static_cast<size_t>(V) * (BF16 ? 2 : 4);
-        double e[2];
-        float2 own[2];
-        float uu[2];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int c = lane + 32 * h;
-          own[h] = c < N ? __ldcg(p.rowstat + brow + c) : make_float2(0.f, 0.f);
-          uu[h] = c < N ? p.uniforms[brow + c] : 1.f;
-          e[h] = 0.0;
-        }
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int c = lane + 32 * h;
-          if (c >= 1 && c < N) {
-            const float2 prs = __ldcg(p.rowstat + brow + par[h]);
-            const float x = load_elem<BF16>(tbase + (brow + par[h]) * rbytes, tok[h]);
-            e[h] = exp((static_cast<double>(x) - prs.x) / static_cast<double>(T));
-          }
-        }
-        bool dup[2] = {false, false};
-        for (int o = 0; o < 64; ++o) {
-          const int t_o = __shfl_sync(0xffffffffu, o < 32 ? tok[0] : tok[1], o & 31);
-          const int p_o = __shfl_sync(0xffffffffu, o < 32 ? par[0] : par[1], o & 31);
-#pragma unroll
-          for (int h = 0; h < 2; ++h) dup[h] |= o < lane + 32 * h && p_o == par[h] && t_o == tok[h];
-        }
-        int live[2];  // a proposal with weight (not a repeat)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          if (dup[h]) e[h] = 0.0;
-          live[h] = e[h] > 0.0 ? 1 : 0;
-        }
-        for (int step = 1; step <= N; ++step) {
-          const float s_cur = __shfl_sync(0xffffffffu, cur < 32 ? own[0].y : own[1].y, cur & 31);
-          bool ch[2], acc[2];
-          double w[2];
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            ch[h] = par[h] == cur;
-            w[h] = ch[h] ? e[h] : 0.0;
-          }
-          // mass removed before each child: exclusive prefix over node order
-          double inc0 = w[0], inc1 = w[1];
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const double y0 = __shfl_up_sync(0xffffffffu, inc0, o);
-            const double y1 = __shfl_up_sync(0xffffffffu, inc1, o);
-            if (lane >= o) { inc0 += y0; inc1 += y1; }
-          }
-          const double tot0 = __shfl_sync(0xffffffffu, inc0, 31);
-          const double ex0 = inc0 - w[0], ex1 = tot0 + inc1 - w[1];
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const double S = static_cast<double>(s_cur) - (h == 0 ? ex0 : ex1);
-            acc[h] = ch[h] && live[h] &&
-                     (S <= w[h] || static_cast<double>(uu[h]) <= w[h] / S);
-          }
-          const unsigned m0 = __ballot_sync(0xffffffffu, acc[0]);
-          const unsigned m1 = __ballot_sync(0xffffffffu, acc[1]);
-          int nxt = -1;
-          if (m0) nxt = __ffs(m0) - 1;
-          else if (m1) nxt = 32 + __ffs(m1) - 1;
-          if (nxt >= 0) {
-            const int t = __shfl_sync(0xffffffffu, nxt < 32 ? tok[0] : tok[1], nxt & 31);
-            if (lane == 0) {
-              path[len] = nxt;
-              out[len] = t;
-            }
-            cur = nxt;
-            ++len;
-            continue;
-          }
-          const float m_cur = __shfl_sync(0xffffffffu, cur < 32 ? own[0].x : own[1].x, cur & 31);
-          const char* crow = tbase + (brow + cur) * rbytes;
-          // every child rejected: hand the final node and its rejected tokens (ascending,
-          // with their weights relative to the row maximum) to the whole block
-          float wrm[2];
-#pragma unroll
-          for (int h = 0; h < 2; ++h)
-            wrm[h] = ch[h] && live[h] ? rel_weight(load_elem<BF16>(crow, tok[h]), m_cur, cs) : 0.f;
-          int rank[2] = {0, 0};
-          for (int o = 0; o < 64; ++o) {
-            const int t_o = __shfl_sync(0xffffffffu, o < 32 ? tok[0] : tok[1], o & 31);
-            const int p_o = __shfl_sync(0xffffffffu, o < 32 ? par[0] : par[1], o & 31);
-            const int l_o = __shfl_sync(0xffffffffu, o < 32 ? live[0] : live[1], o & 31);
-            const bool in = p_o == cur && l_o;
-#pragma unroll
-            for (int h = 0; h < 2; ++h)
-              rank[h] += in && (t_o < tok[h] || (t_o == tok[h] && o < lane + 32 * h));
-          }
-#pragma unroll
-          for (int h = 0; h < 2; ++h)
-            if (ch[h] && live[h]) {
-              s_rm[rank[h]] = tok[h];
-              s_rmw[rank[h]] = wrm[h];
-              s_rmk[rank[h]] = tok[h] / p.elems_per_split;
-            }
-          const int nrm = __popc(__ballot_sync(0xffffffffu, ch[0] && live[0])) +
-                          __popc(__ballot_sync(0xffffffffu, ch[1] && live[1]));
-          if (lane == 0) {
-            s_final = cur;
-            s_len = len;
-            s_nrm = nrm;
-          }
-          break;
-        }
-        for (int c = len + lane; c < N; c += 32) path[c] = -1;
       }
     }
   }
+  int32_t* path = p.path + brow;
+  int32_t* out = p.out_tokens + static_cast<int64_t>(b) * (N + 1);
+  // thread c < N holds node c
+  const int c = tid;
+  const int tok = c < N ? p.tokens[brow + c] : -1, par = c < N ? p.parents[brow + c] : -2;
+  const float uc = tempered && c < N ? p.uniforms[brow + c] : 1.f;
+  if (c < 64) {
+    s_tok_in[c] = tok;
+    s_par[c] = par;
+  }
   __syncthreads();
-  if (s_final < 0) return;  // greedy, bad input: done
+  if (c < N) {
+    uint32_t bad_in = 0;
+    if (tok < 0 || tok >= V) bad_in |= SPEC_FLAG_BAD_TOKEN;
+    if (c == 0 ? par != -1 : (par < 0 || par >= c)) bad_in |= SPEC_FLAG_BAD_TREE;
+    if (s_arg[c] < 0) bad_in |= SPEC_FLAG_BAD_LOGITS;
+    if (bad_in) atomicOr(&s_badin, bad_in);
+  }
+  __syncthreads();
+  if (s_badin) {
+    for (int i = tid; i < N; i += kThreads) path[i] = -1;
+    for (int i = tid; i <= N; i += kThreads) out[i] = -1;
+    if (tid == 0) {
+      p.num_accepted[b] = -1;
+      p.num_emitted[b] = 0;
+      set_status(p.status, s_badin);
+    }
+    return;
+  }
+  // Sampled walk: the children of a node, in node order, are point-mass proposals; child c
+  // is accepted iff u[c] <= p'(token), p' the node's target distribution without the tokens
+  // of the siblings rejected before it. Whether a node is accepted when its turn comes does
+  // not depend on the walk, so every node's test is taken at once, a thread each: its
+  // weight e_c = exp((l(t_c) - M) / T) in fp64 under its parent's row (M that row's
+  // maximum; 0 for a repeated sibling token, removed with its first occurrence), the weight
+  // of its earlier siblings in node order, and u[c] (S - earlier) <= e_c. The walk is then
+  // a ballot per step (with fp64 prefix scans and a division per step, on the one warp
+  // that held the tree, it took 8.7 us of the kernel's 30).
+  const char* tbase = static_cast<const char*>(p.target);
+  const size_t rbytes = static_cast<size_t>(V) * (BF16 ? 2 : 4);
+  bool live = false, acc = false;
+  if (tempered) {
+    const bool child = c >= 1 && c < N;
+    double e = 0.0;
+    if (child) {
+      const float x = load_elem<BF16>(tbase + (brow + par) * rbytes, tok);
+      e = exp((static_cast<double>(x) - s_stat[par].x) / static_cast<double>(T));
+      bool dup = false;
+      for (int o = 1; o < c; ++o) dup |= s_par[o] == par && s_tok_in[o] == tok;
+      if (dup) e = 0.0;
+      s_e[c] = e;
+    }
+    __syncthreads();
+    if (child) {
+      double earlier = 0.0;
+      for (int o = 1; o < c; ++o)
+        if (s_par[o] == par) earlier += s_e[o];
+      live = e > 0.0;
+      const double S = static_cast<double>(s_stat[par].y) - earlier;
+      acc = live && (S <= e || static_cast<double>(uc) * S <= e);
+    }
+  } else {
+    // greedy: a child is accepted iff its token is its parent's argmax
+    acc = c >= 1 && c < N && tok == s_arg[par];
+  }
+  if (c < 64) s_acc[c] = acc ? 1 : 0;
+  __syncthreads();
+  if (tid < 32) {
+    // one warp: lane l holds nodes l and l + 32
+    const int lane = tid;
+    const int par1 = s_par[lane + 32];
+    const bool acc1 = s_acc[lane + 32] != 0;
+    int cur = 0, len = 1;
+    if (lane == 0) {
+      path[0] = 0;
+      out[0] = tok;
+    }
+    for (int step = 1; step < N; ++step) {
+      const unsigned m0 = __ballot_sync(0xffffffffu, par == cur && acc);
+      const unsigned m1 = __ballot_sync(0xffffffffu, par1 == cur && acc1);
+      if (!m0 && !m1) break;
+      cur = m0 ? __ffs(m0) - 1 : 32 + __ffs(m1) - 1;  // the first accepted child in node order
+      if (lane == 0) {
+        path[len] = cur;
+        out[len] = s_tok_in[cur];
+      }
+      ++len;
+    }
+    for (int i = len + lane; i < N; i += 32) path[i] = -1;
+    if (!tempered) {
+      if (lane == 0) {
+        out[len] = s_arg[cur];
+        p.num_accepted[b] = len - 1;
+        p.num_emitted[b] = len + 1;
+      }
+      for (int i = len + 1 + lane; i <= N; i += 32) out[i] = -1;
+    } else if (lane == 0) {  // every child of `cur` rejected: the whole block draws
+      s_final = cur;
+      s_len = len;
+      s_nrm = 0;
+    }
+  }
+  __syncthreads();
+  if (s_final < 0) return;  // greedy: done
+  if (live && par == s_final) {
+    // a rejected token of the final node: its weight relative to the row maximum, its place
+    // among them by token
+    int rank = 0;
+    for (int o = 1; o < N; ++o) rank += s_par[o] == par && s_e[o] > 0.0 && s_tok_in[o] < tok;
+    s_rm[rank] = tok;
+    s_rmw[rank] = rel_weight(load_elem<BF16>(tbase + (brow + par) * rbytes, tok), s_stat[par].x, cs);
+    s_rmk[rank] = tok / p.elems_per_split;
+    atomicAdd(&s_nrm, 1);
+  }
+  __syncthreads();
 
   // ---- the final draw from p' of node s_final: inverse CDF in ascending token order ----
   const int fin = s_final, len = s_len, nrm = s_nrm;
   const int64_t frid = brow + fin;
-  const float M = __ldcg(p.rowstat + frid).x;
+  const float M = s_stat[fin].x;
   const int eps = p.elems_per_split;
   if (tid < 32) {
     // remaining mass of each part (its sum minus its rejected tokens' weights), the total,
@@ -476,8 +391,8 @@ __global__ void __launch_bounds__(kThreads, kTreeBlocksPerSm) tree_greedy_kernel
     const int k = tid;
     double base = 0.0;
     if (k < p.splits) {
-      const uint4 q = __ldcg(p.parts + frid * p.splits + k);
-      base = static_cast<double>(__uint_as_float(q.w)) * rel_weight(key_to_float(q.y), M, cs);
+      const float2 q = s_part[fin * 16 + k];
+      base = static_cast<double>(q.y) * rel_weight(q.x, M, cs);
     }
     double removed = 0.0;
     for (int r = 0; r < nrm; ++r)
@@ -523,29 +438,10 @@ __global__ void __launch_bounds__(kThreads, kTreeBlocksPerSm) tree_greedy_kernel
   const char* frow = static_cast<const char*>(p.target) + frid * V * (BF16 ? 2 : 4);
   int ptr = 0;
   while (ptr < nrm_scan && s_rm[ptr] < lo) ++ptr;
-  // The run is read kChunk elements at a time, all of a chunk's loads issued before any
-  // is used (16-byte vectors when the rows allow: a run starts on a multiple of 8
-  // elements, and hi is a multiple of the vector's elements).
-  constexpr int kChunk = 16;
-  auto load_chunk = [&](int x0, float* lv) {
-    if (VEC) {
-      constexpr int kEpv = BF16 ? 8 : 4;
-#pragma unroll
-      for (int v = 0; v < kChunk / kEpv; ++v) {
-        const int x = x0 + v * kEpv;
-        uint4 raw = make_uint4(0u, 0u, 0u, 0u);
-        if (x < hi) raw = __ldg(reinterpret_cast<const uint4*>(frow + static_cast<int64_t>(x) * (BF16 ? 2 : 4)));
-        const uint32_t wv[4] = {raw.x, raw.y, raw.z, raw.w};
-#pragma unroll
-        for (int q = 0; q < kEpv; ++q)
-          lv[v * kEpv + q] = BF16 ? __uint_as_float((q & 1) ? (wv[q >> 1] & 0xffff0000u) : (wv[q >> 1] << 16))
-                                  : __uint_as_float(wv[q]);
-      }
-    } else {
-#pragma unroll
-      for (int i = 0; i < kChunk; ++i) lv[i] = x0 + i < hi ? load_elem<BF16>(frow, x0 + i) : 0.f;
-    }
-  };
+  // The run is read kBatch 16-byte vectors at a time when the rows allow (a run starts on a
+  // multiple of 8 elements, and hi is a multiple of the vector's elements), all of them in
+  // flight together; the code below is per vector, the batch moving up by one each time.
+  constexpr int kEpv = BF16 ? 8 : 4, kBatch = 8;
   // The weight of element x from its logit l, 0 for a removed token. Elements come in
   // ascending order and the removed tokens are distinct and ascending, so the next one is
   // kept in a register.
@@ -560,12 +456,29 @@ __global__ void __launch_bounds__(kThreads, kTreeBlocksPerSm) tree_greedy_kernel
   float run = 0.f;
   {
     int q = ptr, next_rm = ptr < nrm_scan ? s_rm[ptr] : INT_MAX;
-    for (int x0 = lo; x0 < hi; x0 += kChunk) {
-      float lv[kChunk];
-      load_chunk(x0, lv);
+    for (int x0 = lo; x0 < hi; x0 += kBatch * kEpv) {
+      uint4 raw[kBatch];
 #pragma unroll
-      for (int i = 0; i < kChunk; ++i)
-        if (x0 + i < hi) run += weight_of(x0 + i, lv[i], q, next_rm);
+      for (int v = 0; v < kBatch; ++v) {
+        const int x = x0 + v * kEpv;
+        raw[v] = make_uint4(0u, 0u, 0u, 0u);
+        if (VEC && x < hi) raw[v] = __ldg(reinterpret_cast<const uint4*>(frow + static_cast<int64_t>(x) * (BF16 ? 2 : 4)));
+      }
+#pragma unroll 1
+      for (int x = x0; x < min(hi, x0 + kBatch * kEpv); x += kEpv) {
+        float lv[kEpv];
+        const uint32_t wv[4] = {raw[0].x, raw[0].y, raw[0].z, raw[0].w};
+#pragma unroll
+        for (int i = 0; i < kEpv; ++i)
+          lv[i] = !VEC ? (x + i < hi ? load_elem<BF16>(frow, x + i) : 0.f)
+                  : BF16 ? __uint_as_float((i & 1) ? (wv[i >> 1] & 0xffff0000u) : (wv[i >> 1] << 16))
+                         : __uint_as_float(wv[i]);
+#pragma unroll
+        for (int v = 0; v + 1 < kBatch; ++v) raw[v] = raw[v + 1];
+#pragma unroll
+        for (int i = 0; i < kEpv; ++i)
+          if (x + i < hi) run += weight_of(x + i, lv[i], q, next_rm);
+      }
     }
   }
   // block exclusive scan of the runs' sums; the run that holds the crossing is the last
@@ -592,24 +505,42 @@ __global__ void __launch_bounds__(kThreads, kTreeBlocksPerSm) tree_greedy_kernel
   owner = -1;
   for (int k = 0; k < kThreads / 32; ++k) owner = max(owner, __float_as_int(s_fsum[k]));
   if (tid == owner) {
-    // walk the run: the first token whose cumulative weight reaches the target, else (if
-    // rounding leaves the target above the run) its last positive-weight token
-    double C = excl;
-    int q = ptr, next_rm = ptr < nrm_scan ? s_rm[ptr] : INT_MAX, pick = -1;
+    s_lo = lo;
+    s_hi = hi;
+    s_excl = excl;
+  }
+  __syncthreads();
+  if (owner >= 0 && tid < 32) {
+    // one warp over the owner's run, 32 elements at a time: the first token whose cumulative
+    // weight (fp64) reaches the target, else (if rounding leaves the target above the run)
+    // its last positive-weight token. (One thread adding the weights one by one in fp64
+    // took 3.5 us.)
+    const int rlo = s_lo, rhi = s_hi;
+    double C = s_excl;
+    int pick = -1;
     bool done = false;
-    for (int x0 = lo; x0 < hi && !done; x0 += kChunk) {
-      float lv[kChunk];
-      load_chunk(x0, lv);
-      for (int i = 0; i < kChunk && !done && x0 + i < hi; ++i) {
-        const float w = weight_of(x0 + i, lv[i], q, next_rm);
-        C += static_cast<double>(w);
-        if (w > 0.f) {
-          pick = x0 + i;
-          done = C >= tin;
-        }
+    for (int x0 = rlo; x0 < rhi && !done; x0 += 32) {
+      const int x = x0 + tid;
+      float w = x < rhi ? rel_weight(load_elem<BF16>(frow, x), M, cs) : 0.f;
+      for (int r = 0; r < nrm_scan; ++r)
+        if (s_rm[r] == x) w = 0.f;
+      double incl = static_cast<double>(w);
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const double y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (tid >= o) incl += y;
       }
+      const unsigned hit = __ballot_sync(0xffffffffu, w > 0.f && C + incl >= tin);
+      const unsigned any = __ballot_sync(0xffffffffu, w > 0.f);
+      if (hit) {
+        pick = x0 + __ffs(hit) - 1;
+        done = true;
+      } else if (any) {
+        pick = x0 + 31 - __clz(any);
+      }
+      C += __shfl_sync(0xffffffffu, incl, 31);
     }
-    s_tok = pick;
+    if (tid == 0) s_tok = pick;
   }
   if (owner < 0 && tid == 0) s_tok = s_arg[fin];  // no weight left in fp32: the row maximum
   __syncthreads();
@@ -1407,10 +1338,7 @@ cudaError_t launch_tree_greedy(const spec_tree_accept_args_t& a, const TreeLayou
   p.num_emitted = a.num_emitted;
   p.status = reinterpret_cast<uint32_t*>(ws);
   p.tickets = reinterpret_cast<uint32_t*>(ws + L.tickets);
-  p.row_tickets = reinterpret_cast<uint32_t*>(ws + L.row_tickets);
   p.parts = reinterpret_cast<uint4*>(ws + L.parts);
-  p.argmax = reinterpret_cast<int32_t*>(ws + L.argmax);
-  p.rowstat = reinterpret_cast<float2*>(ws + L.rowstat);
   p.temperature = a.temperature;
   p.uniforms = a.uniforms;
   (void)cudaGetLastError();
