@@ -5,16 +5,15 @@
 //
 // tree_greedy_kernel (tree acceptance): grid (splits, nodes, sequences) of 128-thread
 // blocks. Each block finds the lowest-index argmax of its part of a node's target row
-// and, for a tempered sequence, the part's sum of 2^((l - max) log2e / T); the row's
-// last block (ticket) merges the parts, and the sequence's last block walks the tree
-// from the root. Greedy: to the child whose token is the current node's argmax.
+// and, for a tempered sequence, the part's sum of 2^((l - max) log2e / T); the
+// sequence's last block (ticket) merges the parts of all rows and walks the tree from the
+// root. Greedy: to the child whose token is the current node's argmax.
 // Sampled: the children are tried in node order as point-mass proposals (accepted iff
 // u <= p'(token), p' without the siblings rejected before), decided in fp64 from the
-// gathered logits (every node's weight under its parent's row and its earlier siblings'
-// weight are taken once, before the walk, so a step is a shuffle, a division and two
-// ballots); after the last rejection the block draws the final token from p' by
-// inverse CDF: the part where the remaining mass crosses u x total, from the stored part
-// sums minus the rejected tokens' weights, then one pass over that part.
+// gathered logits; every node's test is taken before the walk, which is a ballot per
+// step. After the last rejection the block draws the final token from p' by inverse CDF:
+// the part where the remaining mass crosses u x total, from the stored part sums minus
+// the rejected tokens' weights, then one pass over that part.
 //
 // tree_compact_kernel: one block per (cache, KV head, sequence) moves the accepted
 // path's key or value rows into consecutive positions after the context.
@@ -311,6 +310,7 @@ __global__ void __launch_bounds__(kThreads, kTreeBlocksPerSm) tree_greedy_kernel
       const float x = load_elem<BF16>(tbase + (brow + par) * rbytes, tok);
       e = exp((static_cast<double>(x) - s_stat[par].x) / static_cast<double>(T));
       bool dup = false;
+#pragma unroll 8
       for (int o = 1; o < c; ++o) dup |= s_par[o] == par && s_tok_in[o] == tok;
       if (dup) e = 0.0;
       s_e[c] = e;
@@ -318,6 +318,7 @@ __global__ void __launch_bounds__(kThreads, kTreeBlocksPerSm) tree_greedy_kernel
     __syncthreads();
     if (child) {
       double earlier = 0.0;
+#pragma unroll 8
       for (int o = 1; o < c; ++o)
         if (s_par[o] == par) earlier += s_e[o];
       live = e > 0.0;
@@ -371,6 +372,7 @@ __global__ void __launch_bounds__(kThreads, kTreeBlocksPerSm) tree_greedy_kernel
     // a rejected token of the final node: its weight relative to the row maximum, its place
     // among them by token
     int rank = 0;
+#pragma unroll 8
     for (int o = 1; o < N; ++o) rank += s_par[o] == par && s_e[o] > 0.0 && s_tok_in[o] < tok;
     s_rm[rank] = tok;
     s_rmw[rank] = rel_weight(load_elem<BF16>(tbase + (brow + par) * rbytes, tok), s_stat[par].x, cs);
@@ -442,17 +444,6 @@ __global__ void __launch_bounds__(kThreads, kTreeBlocksPerSm) tree_greedy_kernel
   // multiple of 8 elements, and hi is a multiple of the vector's elements), all of them in
   // flight together; the code below is per vector, the batch moving up by one each time.
   constexpr int kEpv = BF16 ? 8 : 4, kBatch = 8;
-  // The weight of element x from its logit l, 0 for a removed token. Elements come in
-  // ascending order and the removed tokens are distinct and ascending, so the next one is
-  // kept in a register.
-  auto weight_of = [&](int x, float l, int& q, int& next_rm) {
-    if (x == next_rm) {
-      ++q;
-      next_rm = q < nrm_scan ? s_rm[q] : INT_MAX;
-      return 0.f;
-    }
-    return rel_weight(l, M, cs);
-  };
   float run = 0.f;
   {
     int q = ptr, next_rm = ptr < nrm_scan ? s_rm[ptr] : INT_MAX;
@@ -466,7 +457,9 @@ __global__ void __launch_bounds__(kThreads, kTreeBlocksPerSm) tree_greedy_kernel
       }
 #pragma unroll 1
       for (int x = x0; x < min(hi, x0 + kBatch * kEpv); x += kEpv) {
-        float lv[kEpv];
+        // the vector's weights, then the removed tokens' cleared (elements come in ascending
+        // order and the removed tokens are distinct and ascending: the next one is kept)
+        float lv[kEpv], w[kEpv];
         const uint32_t wv[4] = {raw[0].x, raw[0].y, raw[0].z, raw[0].w};
 #pragma unroll
         for (int i = 0; i < kEpv; ++i)
@@ -476,8 +469,16 @@ __global__ void __launch_bounds__(kThreads, kTreeBlocksPerSm) tree_greedy_kernel
 #pragma unroll
         for (int v = 0; v + 1 < kBatch; ++v) raw[v] = raw[v + 1];
 #pragma unroll
-        for (int i = 0; i < kEpv; ++i)
-          if (x + i < hi) run += weight_of(x + i, lv[i], q, next_rm);
+        for (int i = 0; i < kEpv; ++i) w[i] = x + i < hi ? rel_weight(lv[i], M, cs) : 0.f;
+        while (next_rm < x + kEpv) {
+#pragma unroll
+          for (int i = 0; i < kEpv; ++i)
+            if (x + i == next_rm) w[i] = 0.f;
+          ++q;
+          next_rm = q < nrm_scan ? s_rm[q] : INT_MAX;
+        }
+#pragma unroll
+        for (int i = 0; i < kEpv; ++i) run += w[i];
       }
     }
   }
@@ -811,106 +812,113 @@ __device__ __forceinline__ unsigned long long block_max_u64(unsigned long long v
 // about 48 bits this way without fp64 arithmetic, whose latency is high on this part.
 __device__ __forceinline__ void df_add(float ah, float al, float b, float& rh, float& rl) {
   const float s = __fadd_rn(ah, b);
-  if (!(s > -INFINITY)) {  // a -inf term
-    rh = s;
-    rl = 0.f;
-    return;
-  }
   const float bb = __fsub_rn(s, ah);
   const float e = __fadd_rn(__fsub_rn(ah, __fsub_rn(s, bb)), __fsub_rn(b, bb));
   const float t = __fadd_rn(e, al);
-  rh = __fadd_rn(s, t);
-  rl = __fsub_rn(t, __fsub_rn(rh, s));
+  const float h = __fadd_rn(s, t);
+  const bool none = !(s > -INFINITY);  // a -inf term
+  rh = none ? s : h;
+  rl = none ? 0.f : __fsub_rn(t, __fsub_rn(h, s));
 }
 
 struct TreeNode {
-  int dep, nx, tok, par;   // dep < 0: no node in this slot
+  int dep, nx, par, idx;   // dep < 0: no node in this slot; idx: the parent's candidate it took
   float sh, sl;            // path score as an unevaluated sum sh + sl (double-float)
-  float oh, ol;            // score of the current offer, the same way
-  int otk;                 // token of the current offer
-  unsigned long long key;  // order key of the offer's score, 0 if none
+  // Scores the node may bring to the next steps, the same way, each with the order key of its
+  // high part (0 if there is none): its current offer (candidate nx of position dep + 1), the
+  // offer after that, and the first offer of the node the current one would become.
+  float oh, ol, nh, nl, ch, cl;
+  uint32_t ok, nk, ck;
+  float nq, cq;            // log q of the last two, read ahead; NaN: there is none
   unsigned long long msk;  // ancestor bits
 };
 
-// The node's next offer, its candidate nx of position dep + 1 (table row dep): its score
-// (oh + ol) and token, and the key (0 if there is none) that orders normalised
-// double-floats: high parts first, then low parts.
-__device__ __forceinline__ unsigned long long offer_of(const TreeNode& n, const int2* tab, int rows, int K,
-                                                       float& oh, float& ol, int& otk) {
-  if (n.dep < 0 || n.dep >= rows || n.nx >= K) return 0ull;
-  const int2 e = tab[n.dep * K + n.nx];
-  df_add(n.sh, n.sl, __int_as_float(e.y), oh, ol);
-  otk = e.x;
-  return (static_cast<unsigned long long>(order_key(oh)) << 32) | order_key(ol);
-}
-
 // Best-first selection of the tree's nodes by one warp. The root (node 0) is kept in
 // every lane; node c >= 1 is slot (c - 1) / 32 of lane (c - 1) % 32. Each step takes the
-// best offer (largest high word of its key; on a tie the largest low word, then the
-// lowest node index, the root first), makes it node i, and moves its parent to its next
-// candidate.
+// best offer (largest high part; on a tie the largest low part, then the lowest node
+// index, the root first), makes it node i, and moves its parent to its next candidate.
+// Both of the offers a step puts up were scored when the one it takes was, so a step's
+// chain is a warp maximum, a ballot and a shuffle, and the table is read beside it
+// (scored within the step and with branches: 0.37 us a node, now 0.24; tokens follow from
+// the parents' candidates at the end).
 template <int SLOTS>
 __device__ __forceinline__ void select_nodes(const BuildParams& p, const int2* tab, int K, int b,
                                              uint32_t flags, int lane) {
   const int N = p.nodes;
   const int64_t base = static_cast<int64_t>(b) * N;
-  TreeNode root, n[SLOTS];
-  root.dep = 0;
-  root.nx = 0;
-  root.tok = flags ? -1 : p.root[b];
+  // log q of candidate nx of table row dep (NaN past the table), without a branch
+  auto cand_q = [&](int dep, int nx) -> float {
+    const bool valid = static_cast<unsigned>(dep) < static_cast<unsigned>(p.rows) && nx < K;
+    const float q = __int_as_float(tab[valid ? dep * K + nx : 0].y);
+    return valid ? q : NAN;
+  };
+  // the reads of the node's next offers, and their scores from what was read
+  auto fetch = [&](TreeNode& n) {
+    n.nq = cand_q(n.dep, n.nx + 1);
+    n.cq = cand_q(n.ok ? n.dep + 1 : -1, 0);
+  };
+  auto score = [&](TreeNode& n) {
+    df_add(n.sh, n.sl, n.nq, n.nh, n.nl);
+    df_add(n.oh, n.ol, n.cq, n.ch, n.cl);
+    n.nk = n.nq == n.nq ? order_key(n.nh) : 0u;
+    n.ck = n.cq == n.cq ? order_key(n.ch) : 0u;
+  };
+  TreeNode root = {}, n[SLOTS];
   root.par = -1;
   root.msk = 1ull;
-  root.sh = root.sl = 0.f;
-  root.oh = root.ol = 0.f;
-  root.otk = -1;
-  root.key = 0ull;
 #pragma unroll
   for (int h = 0; h < SLOTS; ++h) {
+    n[h] = {};
     n[h].dep = -1;
-    n[h].nx = 0;
-    n[h].tok = -1;
     n[h].par = -1;
-    n[h].msk = 0ull;
-    n[h].sh = n[h].sl = 0.f;
-    n[h].oh = n[h].ol = 0.f;
-    n[h].otk = -1;
-    n[h].key = 0ull;
   }
   if (!flags) {
-    root.key = offer_of(root, tab, p.rows, K, root.oh, root.ol, root.otk);
+    const float q0 = cand_q(0, 0);
+    df_add(0.f, 0.f, q0, root.oh, root.ol);
+    root.ok = q0 == q0 ? order_key(root.oh) : 0u;
+    fetch(root);
+    score(root);
+#pragma unroll
+    for (int h = 0; h < SLOTS; ++h) fetch(n[h]);
+#pragma unroll 1
     for (int i = 1; i < N; ++i) {
-      const uint32_t rh = static_cast<uint32_t>(root.key >> 32);
       uint32_t hl = 0u;
 #pragma unroll
-      for (int h = 0; h < SLOTS; ++h) hl = max(hl, static_cast<uint32_t>(n[h].key >> 32));
-      const uint32_t Mh = max(__reduce_max_sync(0xffffffffu, hl), rh);
+      for (int h = 0; h < SLOTS; ++h) hl = max(hl, n[h].ok);
+      const uint32_t Mh = max(__reduce_max_sync(0xffffffffu, hl), root.ok);
+#pragma unroll
+      for (int h = 0; h < SLOTS; ++h) score(n[h]);  // beside the maximum's latency
       if (Mh == 0u) {  // no offer left: excluded by the host's capacity check
         flags |= SPEC_FLAG_BAD_TREE;
         break;
       }
       unsigned bal[SLOTS];
-      int ties = rh == Mh;
+      int ties = root.ok == Mh;
 #pragma unroll
       for (int h = 0; h < SLOTS; ++h) {
-        bal[h] = __ballot_sync(0xffffffffu, static_cast<uint32_t>(n[h].key >> 32) == Mh);
+        bal[h] = __ballot_sync(0xffffffffu, n[h].ok == Mh);
         ties += __popc(bal[h]);
       }
-      bool root_wins = rh == Mh;
+      bool root_wins = root.ok == Mh;
       if (ties > 1) {
-        const uint32_t rl = rh == Mh ? static_cast<uint32_t>(root.key) : 0u;
+        const uint32_t rl = root.ok == Mh ? order_key(root.ol) : 0u;
         uint32_t ll = 0u;
 #pragma unroll
         for (int h = 0; h < SLOTS; ++h)
-          if (static_cast<uint32_t>(n[h].key >> 32) == Mh) ll = max(ll, static_cast<uint32_t>(n[h].key));
+          if (n[h].ok == Mh) ll = max(ll, order_key(n[h].ol));
         const uint32_t Ml = max(__reduce_max_sync(0xffffffffu, ll), rl);
-        root_wins = rh == Mh && rl == Ml;
+        root_wins = root.ok == Mh && rl == Ml;
 #pragma unroll
         for (int h = 0; h < SLOTS; ++h)
-          bal[h] = __ballot_sync(0xffffffffu, static_cast<uint32_t>(n[h].key >> 32) == Mh &&
-                                                  static_cast<uint32_t>(n[h].key) == Ml);
+          bal[h] = __ballot_sync(0xffffffffu, n[h].ok == Mh && order_key(n[h].ol) == Ml);
       }
-      // the winner u and its offer (score, token), depth and ancestor bits
+      // the winner u, its offer and that offer's own first offer, depth and ancestor bits
       int u = 0, hs = 0;
+      float wh = root.oh, wl = root.ol, wch = root.ch, wcl = root.cl;
+      uint32_t wck = root.ck;
+      int wdn = root.nx;  // depth << 16 | candidate
+      unsigned long long wm = 1ull;
+      int src = 0;
       if (!root_wins) {
 #pragma unroll
         for (int h = SLOTS - 1; h >= 0; --h)
@@ -918,71 +926,55 @@ __device__ __forceinline__ void select_nodes(const BuildParams& p, const int2* t
             u = 1 + 32 * h + __ffs(bal[h]) - 1;
             hs = h;
           }
-      }
-      const int src = (u - 1) & 31;
-      float oh = root.oh, ol = root.ol;
-      int otk = root.otk, pdep = 0;
-      unsigned long long pm = 1ull;
-      {
-        float soh = n[0].oh, sol = n[0].ol;
-        int sotk = n[0].otk, sdep = n[0].dep;
-        unsigned long long smsk = n[0].msk;
-#pragma unroll
-        for (int h = 1; h < SLOTS; ++h)
-          if (hs == h) {
-            soh = n[h].oh;
-            sol = n[h].ol;
-            sotk = n[h].otk;
-            sdep = n[h].dep;
-            smsk = n[h].msk;
-          }
-        soh = __shfl_sync(0xffffffffu, soh, src);
-        sol = __shfl_sync(0xffffffffu, sol, src);
-        sotk = __shfl_sync(0xffffffffu, sotk, src);
-        sdep = __shfl_sync(0xffffffffu, sdep, src);
-        smsk = __shfl_sync(0xffffffffu, smsk, src);
-        if (u != 0) {
-          oh = soh;
-          ol = sol;
-          otk = sotk;
-          pdep = sdep;
-          pm = smsk;
-        }
+        src = (u - 1) & 31;
+        constexpr int L = SLOTS - 1;
+        const bool up = SLOTS > 1 && hs == L;
+        wck = __shfl_sync(0xffffffffu, up ? n[L].ck : n[0].ck, src);
+        wch = __shfl_sync(0xffffffffu, up ? n[L].ch : n[0].ch, src);
+        wcl = __shfl_sync(0xffffffffu, up ? n[L].cl : n[0].cl, src);
+        wh = __shfl_sync(0xffffffffu, up ? n[L].oh : n[0].oh, src);
+        wl = __shfl_sync(0xffffffffu, up ? n[L].ol : n[0].ol, src);
+        wdn = __shfl_sync(0xffffffffu, up ? (n[L].dep << 16) | n[L].nx : (n[0].dep << 16) | n[0].nx, src);
+        wm = __shfl_sync(0xffffffffu, up ? n[L].msk : n[0].msk, src);
       }
       // node i takes the offer; its parent moves to its next candidate
-      const int ci = (i - 1) & 31, ch = (i - 1) >> 5;
+      const int ci = (i - 1) & 31, chs = (i - 1) >> 5;
 #pragma unroll
       for (int h = 0; h < SLOTS; ++h) {
-        const bool is_new = lane == ci && ch == h;
+        const bool is_new = lane == ci && chs == h;
         const bool adv = u != 0 && lane == src && hs == h;
         if (is_new) {
-          n[h].dep = pdep + 1;
+          n[h].dep = (wdn >> 16) + 1;
           n[h].nx = 0;
-          n[h].tok = otk;
           n[h].par = u;
-          n[h].sh = oh;
-          n[h].sl = ol;
-          n[h].msk = pm | (1ull << i);
+          n[h].idx = wdn & 0xffff;
+          n[h].sh = wh;
+          n[h].sl = wl;
+          n[h].oh = wch;
+          n[h].ol = wcl;
+          n[h].ok = wck;
+          n[h].msk = wm | (1ull << i);
         }
-        if (adv) ++n[h].nx;
-        float ph = 0.f, pl = 0.f;
-        int pt = -1;
-        const unsigned long long k = offer_of(n[h], tab, p.rows, K, ph, pl, pt);
-        if (is_new || adv) {
-          n[h].key = k;
-          n[h].oh = ph;
-          n[h].ol = pl;
-          n[h].otk = pt;
+        if (adv) {
+          ++n[h].nx;
+          n[h].oh = n[h].nh;
+          n[h].ol = n[h].nl;
+          n[h].ok = n[h].nk;
         }
+        fetch(n[h]);
       }
       if (u == 0) {
         ++root.nx;
-        root.key = offer_of(root, tab, p.rows, K, root.oh, root.ol, root.otk);
+        root.oh = root.nh;
+        root.ol = root.nl;
+        root.ok = root.nk;
+        fetch(root);
+        score(root);
       }
     }
   }
   if (lane == 0) {
-    p.tokens[base] = flags ? -1 : root.tok;
+    p.tokens[base] = flags ? -1 : p.root[b];
     p.parents[base] = -1;
     if (p.depth) p.depth[base] = flags ? -1 : 0;
     if (p.mask) p.mask[base] = flags ? 0ull : 1ull;
@@ -991,7 +983,7 @@ __device__ __forceinline__ void select_nodes(const BuildParams& p, const int2* t
   for (int h = 0; h < SLOTS; ++h) {
     const int c = 1 + lane + 32 * h;
     if (c >= N) continue;
-    p.tokens[base + c] = flags ? -1 : n[h].tok;
+    p.tokens[base + c] = flags ? -1 : tab[(n[h].dep - 1) * K + n[h].idx].x;
     p.parents[base + c] = flags ? -1 : n[h].par;
     if (p.depth) p.depth[base + c] = flags ? -1 : n[h].dep;
     if (p.mask) p.mask[base + c] = flags ? 0ull : n[h].msk;
