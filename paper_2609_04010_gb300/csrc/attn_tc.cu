@@ -590,26 +590,35 @@ __global__ void __launch_bounds__(TcCfg<D, MT, QR, HP>::THREADS, 1)
         tc_fence_before();
         __syncwarp();
         if (lane == 0 && !C::PTMEM) mbar_arrive(s_free(mt, x & 1));
-        // scale to base 2 and mask keys past ctx + j
+        // mask keys past ctx + j, in the tiles that reach the block's own keys (a whole warp at
+        // a time: with the test per score in every tile, and separate scaling and
+        // subtraction, the softmax took 480 instructions a warp and tile, now about 250)
         const int key0 = (s.tile0 + k) * TK + hf * KH;
-        const int lim = ctx + ro.j - key0;  // keys c <= lim are visible
-        float tmax = -INFINITY;
-        if (TREE) {
-          const int rel0 = key0 - ctx;  // block position of element 0 (negative: the prefix)
+        if (key0 + KH > ctx) {
+          if (TREE) {
+            const int rel0 = key0 - ctx;  // block position of element 0 (negative: the prefix)
 #pragma unroll
-          for (int c = 0; c < KH; ++c) {
-            const int rel = rel0 + c;
-            const bool vis = rel < 0 || (rel < 64 && ((tmask >> rel) & 1ull));
-            v[c] = vis ? v[c] * p.scale_log2 : -INFINITY;
-            tmax = fmaxf(tmax, v[c]);
-          }
-        } else {
+            for (int c = 0; c < KH; ++c) {
+              const int rel = rel0 + c;
+              const bool vis = rel < 0 || (rel < 64 && ((tmask >> rel) & 1ull));
+              if (!vis) v[c] = -INFINITY;
+            }
+          } else {
+            const int lim = ctx + ro.j - key0;  // keys c <= lim are visible
 #pragma unroll
-          for (int c = 0; c < KH; ++c) {
-            v[c] = c <= lim ? v[c] * p.scale_log2 : -INFINITY;
-            tmax = fmaxf(tmax, v[c]);
+            for (int c = 0; c < KH; ++c)
+              if (c > lim) v[c] = -INFINITY;
           }
         }
+        float mx[KH / 4];
+#pragma unroll
+        for (int c = 0; c < KH / 4; ++c)
+          mx[c] = fmaxf(fmaxf(v[c], v[c + KH / 4]), fmaxf(v[c + KH / 2], v[c + 3 * KH / 4]));
+#pragma unroll
+        for (int o = KH / 8; o > 0; o >>= 1)
+#pragma unroll
+          for (int c = 0; c < o; ++c) mx[c] = fmaxf(mx[c], mx[c + o]);
+        const float tmax = mx[0] * p.scale_log2;  // base 2
         const float m_new = fmaxf(m, tmax);
         const bool want = k > 0 && m_new > m + 8.f;
         const bool rescale = __any_sync(0xffffffffu, want);
@@ -622,14 +631,20 @@ __global__ void __launch_bounds__(TcCfg<D, MT, QR, HP>::THREADS, 1)
         }
         const float msub = m == -INFINITY ? 0.f : m;
         uint32_t pk[KH / 2];
-        float sum = 0.f;
+        const uint64_t sc2 = pack2(p.scale_log2, p.scale_log2), ms2 = pack2(-msub, -msub);
+        uint64_t sum[2] = {pack2(0.f, 0.f), pack2(0.f, 0.f)};
 #pragma unroll
         for (int c = 0; c < KH / 2; ++c) {
-          const float a = ex2(v[2 * c] - msub), b2 = ex2(v[2 * c + 1] - msub);
-          sum += a + b2;
+          float a, b2;
+          unpack2(fma2(pack2(v[2 * c], v[2 * c + 1]), sc2, ms2), a, b2);
+          a = ex2(a);
+          b2 = ex2(b2);
+          sum[c & 1] = add2(sum[c & 1], pack2(a, b2));
           pk[c] = pack_bf16(a, b2);
         }
-        l = l * alpha + sum;
+        float s_lo, s_hi;
+        unpack2(add2(sum[0], sum[1]), s_lo, s_hi);
+        l = l * alpha + (s_lo + s_hi);
         const int pbuf = static_cast<int>(x % PB);
         if (k >= PB) {  // the P V that last read this P buffer is complete
           ok = mbar_wait(pv_done(mt, pbuf), ((x - PB) / PB) & 1, abort_flag, p.status);

@@ -312,6 +312,26 @@ __device__ __forceinline__ float reduce8(float* v, int i, Op op) {
   for (int o = 8; o < G; o <<= 1) r = op(r, __shfl_xor_sync(0xffffffffu, r, o));
   return r;
 }
+// Two fp32 operations in one instruction (the packed forms).
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
 // Programmatic dependent launch: let the next kernel on the stream start now / wait for
 // the kernel this one depends on (no-ops for kernels launched without the attribute).
 __device__ __forceinline__ void pdl_launch_dependents() {

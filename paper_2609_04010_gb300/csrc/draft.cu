@@ -125,16 +125,6 @@ __device__ __forceinline__ uint32_t max2(uint32_t a, uint32_t b) {
   const __nv_bfloat162 h = __hmax2(*reinterpret_cast<const __nv_bfloat162*>(&a), *reinterpret_cast<const __nv_bfloat162*>(&b));
   return *reinterpret_cast<const uint32_t*>(&h);
 }
-// Two fp32 multiply-adds in one instruction (the packed form).
-__device__ __forceinline__ void fma2(float a0, float a1, float b, float c, float& d0, float& d1) {
-  uint64_t va, vb, vc, vd;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(va) : "f"(a0), "f"(a1));
-  asm("mov.b64 %0, {%1, %1};" : "=l"(vb) : "f"(b));
-  asm("mov.b64 %0, {%1, %1};" : "=l"(vc) : "f"(c));
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(vd) : "l"(va), "l"(vb), "l"(vc));
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(d0), "=f"(d1) : "l"(vd));
-}
-
 // The reverse: every thread of the group gets all 8 of reduce8's results.
 __device__ __forceinline__ void gather8(float r, int i, float* v) {
   const bool b0 = i & 1, b1 = i & 2, b2 = i & 4;
@@ -227,7 +217,7 @@ __device__ __forceinline__ void scan_bf16(const uint4* dv, int v0, int vend, int
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       float e0, e1;
-      fma2(lo_f(wv[q]), hi_f(wv[q]), c, nlc, e0, e1);
+      unpack2(fma2(pack2(lo_f(wv[q]), hi_f(wv[q])), pack2(c, c), pack2(nlc, nlc)), e0, e1);
       sum += ex2(e0);
       sum += ex2(e1);
     }

@@ -199,26 +199,6 @@ struct RowStats {
   float z;   // 0, or NaN after a NaN or an infinity
 };
 
-// Two fp32 operations in one instruction (the packed forms).
-__device__ __forceinline__ uint64_t pack2(float a, float b) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ void unpack2(uint64_t v, float& a, float& b) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-
 // W logits of this thread's row, at vocabulary indices col0.., of which the first nv are
 // real, folded into its statistics. About 3.5 instructions a logit: a tree of maxima, one
 // packed multiply-add for the non-finite test (x * 0 is NaN for NaN and infinities), one
