@@ -411,16 +411,17 @@ __global__ void __launch_bounds__(TcCfg<D, MT, QR, HP>::THREADS, 1)
                        : mbar_wait(kv_full(st), (x / C::STAGES) & 1, abort_flag, p.status);
           if (!ok) break;
           if (HP == 1) zero_v_tail(st, s, k);  // the stage's V has landed with its K
-          // S[x & 1] is free once tile x - 2's softmax has read it (and, with P in TMEM,
-          // once that tile's P V MMAs have read its P)
-          if (x >= 2)
-            for (int mt = 0; mt < MT && ok; ++mt)
-              ok = mbar_wait(C::PTMEM ? pv_done(mt, x & 1) : s_free(mt, x & 1), ((x >> 1) - 1) & 1,
-                             abort_flag, p.status);
-          if (!ok) break;
-          tc_fence_after();
-          if (lane == 0) {
-            for (int mt = 0; mt < MT; ++mt) {
+          // One M tile at a time: its S[x & 1] is free once tile x - 2's softmax has read it
+          // (and, with P in TMEM, once that tile's P V MMAs have read its P). The M tiles
+          // then take turns on the tensor pipe instead of waiting for one another
+          // (in step: 147 us for 4 x 32,768 keys at 256 rows, now 141).
+          for (int mt = 0; mt < MT && ok; ++mt) {
+            if (x >= 2)
+              ok = mbar_wait(C::PTMEM ? pv_done(mt, x & 1) : s_free(mt, x & 1), ((x >> 1) - 1) & 1, abort_flag,
+                             p.status);
+            if (!ok) break;
+            tc_fence_after();
+            if (lane == 0) {
 #pragma unroll
               for (int h = 0; h < HP; ++h) {
                 const uint32_t d_tmem = tmem + C::S_COL + ((mt * HP + h) * 2 + (x & 1)) * TK;
@@ -433,10 +434,12 @@ __global__ void __launch_bounds__(TcCfg<D, MT, QR, HP>::THREADS, 1)
                 }
               }
               mma_commit(s_full(mt, x & 1));
+              issued = true;
             }
-            if (HP == 2) mma_commit(k_empty(st));
-            issued = true;
+            __syncwarp();
           }
+          if (!ok) break;
+          if (HP == 2 && lane == 0) mma_commit(k_empty(st));
           __syncwarp();
           if (p.q_tma && k == s.ntile - 1 && has_more(s, t1, OVH)) {
             // the segment's last scores are done with its Q tile: fetch the next one
@@ -455,12 +458,11 @@ __global__ void __launch_bounds__(TcCfg<D, MT, QR, HP>::THREADS, 1)
             zero_v_tail(st, s, k);
           }
           const int pbuf = static_cast<int>(x % PB);
-          for (int mt = 0; mt < MT && ok; ++mt)
+          for (int mt = 0; mt < MT && ok; ++mt) {
             ok = mbar_wait(p_full(mt, pbuf), (x / PB) & 1, abort_flag, p.status);
-          if (!ok) break;
-          tc_fence_after();
-          if (lane == 0) {
-            for (int mt = 0; mt < MT; ++mt) {
+            if (!ok) break;
+            tc_fence_after();
+            if (lane == 0) {
 #pragma unroll
               for (int h = 0; h < HP; ++h) {
 #pragma unroll
@@ -483,10 +485,12 @@ __global__ void __launch_bounds__(TcCfg<D, MT, QR, HP>::THREADS, 1)
                 }
               }
               mma_commit(pv_done(mt, pbuf));
+              issued = true;
             }
-            mma_commit(HP == 2 ? v_empty(st) : kv_empty(st));
-            issued = true;
+            __syncwarp();
           }
+          if (!ok) break;
+          if (lane == 0) mma_commit(HP == 2 ? v_empty(st) : kv_empty(st));
           __syncwarp();
         }
       }
