@@ -233,10 +233,16 @@ __global__ void __launch_bounds__(kStatsThreads, 5) row_stats_kernel(AcceptParam
       const char* at = from - off + static_cast<int64_t>(h0) * E;
       const int ngran = (min(kHalf, len - h0) * E + static_cast<int>(off) + 15) / 16;
       uint4 g[kGran / 32];
+      // one test for all of a lane's loads where the values are 16-bit; with fp32 its second
+      // copy of the loads spills (32.8 us instead of 28.6 on 112 + 80 rows of 50,257)
+      if constexpr (BF16) {
+        load_granules<E, kGran / 32>(g, at, lane, 32, min(ngran, kGran - 1), lo, hi);
+      } else {
 #pragma unroll
-      for (int i = 0; i < kGran / 32; ++i) {
-        const int j = i * 32 + lane;
-        g[i] = j < ngran ? load_granule<E>(at + 16 * j, lo, hi) : make_uint4(0, 0, 0, 0);
+        for (int i = 0; i < kGran / 32; ++i) {
+          const int j = i * 32 + lane;
+          g[i] = j < ngran ? load_granule<E>(at + 16 * j, lo, hi) : make_uint4(0, 0, 0, 0);
+        }
       }
       const uint4 last = kGran - 1 < ngran ? load_granule<E>(at + 16 * (kGran - 1), lo, hi) : make_uint4(0, 0, 0, 0);
       __syncwarp();  // the previous half has been read
@@ -340,10 +346,11 @@ __device__ __forceinline__ void load_run(const void* row, int first, const char*
   } else {
     const uint32_t off = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(a)) & 15u;  // the same for a whole row
     a -= off;
+    uint4 v[NG + 1];
+    load_granules<E, NG + 1>(v, a, 0, 1, off > 0 ? NG + 1 : NG, lo, hi);
 #pragma unroll
     for (int g = 0; g <= NG; ++g) {
-      const uint4 v = g < NG || off > 0 ? load_granule<E>(a + 16 * g, lo, hi) : make_uint4(0, 0, 0, 0);
-      w[4 * g] = v.x; w[4 * g + 1] = v.y; w[4 * g + 2] = v.z; w[4 * g + 3] = v.w;
+      w[4 * g] = v[g].x; w[4 * g + 1] = v[g].y; w[4 * g + 2] = v[g].z; w[4 * g + 3] = v[g].w;
     }
     if (off & 8u) {
 #pragma unroll

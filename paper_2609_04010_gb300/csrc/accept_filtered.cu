@@ -773,11 +773,7 @@ __global__ void __launch_bounds__(kRowThreads, 8) filter_row_kernel(FiltParams p
       const uint32_t off = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(from)) & 15u;
       const int ngran = (min(kStage, e_end - h0) * E + static_cast<int>(off) + 15) / 16;
       uint4 g[kStageGranules / kRowThreads];
-#pragma unroll
-      for (int k = 0; k < kStageGranules / kRowThreads; ++k) {
-        const int n = k * kRowThreads + tid;
-        g[k] = n < ngran ? load_granule<E>(from - off + 16 * n, lo, hi) : make_uint4(0, 0, 0, 0);
-      }
+      load_granules<E, kStageGranules / kRowThreads>(g, from - off, tid, kRowThreads, min(ngran, kStageGranules), lo, hi);
       const uint4 last = tid == 0 && ngran > kStageGranules
                              ? load_granule<E>(from - off + 16 * kStageGranules, lo, hi) : make_uint4(0, 0, 0, 0);
       __syncthreads();  // the previous stage has been read

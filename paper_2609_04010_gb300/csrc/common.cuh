@@ -290,6 +290,32 @@ __device__ __forceinline__ uint4 load_granule(const char* a, const char* lo, con
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
+// Granules n = first, first + stride, .. below `count` from `at` (N of them a thread, zeros
+// past the count) of a tensor [lo, hi): whole loads without a test each where all of them
+// lie inside, which is everywhere but at the tensor's ends (a test for each load: the
+// acceptance of 32 x 8 rows of 100,003 bf16 logits took 48.9 us instead of 45.2, the block
+// draws 57.1 instead of 55.3, filtered rows of 50,257 fp32 logits 28.9 instead of 28.3).
+template <int E, int N>
+__device__ __forceinline__ void load_granules(uint4* g, const char* at, int first, int stride, int count,
+                                              const char* lo, const char* hi) {
+  if (at >= lo && at + 16 * static_cast<int64_t>(count) <= hi) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const int n = first + i * stride;
+      g[i] = n < count ? __ldg(reinterpret_cast<const uint4*>(at) + n) : make_uint4(0u, 0u, 0u, 0u);
+    }
+  } else {
+#pragma unroll 1
+    for (int i = 0; i < N; ++i) {
+      const int n = first + i * stride;
+      const uint4 v = n < count ? load_granule<E>(at + 16 * n, lo, hi) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+      for (int k = 0; k < N; ++k)
+        if (k == i) g[k] = v;
+    }
+  }
+}
+
 // Reduction of 8 values over the threads of a group of G, all 8 together: the tree of a
 // butterfly (neighbours first), but each of the first three exchanges halves the values a
 // thread carries, 7 to 9 shuffles instead of 8 log2 G. Thread i of the group gets value

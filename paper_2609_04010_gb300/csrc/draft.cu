@@ -349,11 +349,7 @@ __global__ void __launch_bounds__(kThreads, 8) draft_sample_kernel(DraftParams p
       const uint32_t off = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(from)) & 15u;
       const int ngran = (min(kStage, e_end - h0) * E + static_cast<int>(off) + 15) / 16;
       uint4 g[kStageGranules / kThreads];
-#pragma unroll
-      for (int k = 0; k < kStageGranules / kThreads; ++k) {
-        const int n = k * kThreads + tid;
-        g[k] = n < ngran ? load_granule<E>(from - off + 16 * n, lo, hi) : make_uint4(0, 0, 0, 0);
-      }
+      load_granules<E, kStageGranules / kThreads>(g, from - off, tid, kThreads, min(ngran, kStageGranules), lo, hi);
       const uint4 last = tid == 0 && ngran > kStageGranules
                              ? load_granule<E>(from - off + 16 * kStageGranules, lo, hi) : make_uint4(0, 0, 0, 0);
       __syncthreads();  // the previous stage has been read
