@@ -311,6 +311,8 @@ def attn_path_name(choice, binding, ai):
     """The attention kernel the library picks for this workload and --attn-path."""
     group = ai.num_q_heads // ai.num_kv_heads
     rows = group * ai.gamma
+    if choice == "auto" and rows <= 32 and ai.num_kv_heads % 2 == 0:
+        return "tensor cores, groups of KV heads"
     if choice == "auto":
         choice = "tensor-cores" if rows >= binding.tensor_core_min_rows() else "cuda-cores"
     if choice == "keys-on-lanes":
@@ -319,6 +321,14 @@ def attn_path_name(choice, binding, ai):
     if choice == "tensor-cores":
         return "tensor cores, row tiles"
     return choice.replace("-", " ")
+
+
+def launches_per_step(path, filtered):
+    """Kernels of one verify step: attention (with a merge kernel behind it, but for the two
+    paths that merge in the kernel), then row statistics, decisions and draws, or the one
+    filtered acceptance kernel. The bench's contexts are all long enough to be split."""
+    merge = path not in ("cuda cores", "tensor cores, keys on lanes")
+    return 1 + int(merge) + (1 if filtered else 3)
 
 
 class StepSetup:
@@ -546,9 +556,6 @@ def run_ours(args, wl, ai, ci, rank, world, local_rank):
     dom_bytes = tm["kv"] if dominant == "attention" else tm["logits"]
     dom_ms = attn_ms if dominant == "attention" else acc_ms
     dom_gbs = dom_bytes / (dom_ms / 1000.0) / 1e9
-    # attention, then row statistics, decisions, draws; a filtered step: attention and
-    # the one filtered acceptance kernel
-    launches_per_step = 2 if filtered else 4
     traffic, traffic_src = (None, None)
     if dominant == "attention" and attn_path_name(args.attn_path, binding, ai) == "tensor cores, row tiles":
         traffic, traffic_src = measured_traffic(args.workload, "attention")
@@ -574,7 +581,7 @@ def run_ours(args, wl, ai, ci, rank, world, local_rank):
                           "frac_of_8tbs": round(step_gbs / NOMINAL_HBM_GBS, 4)},
         "parts_ms": {"attention": attn_ms, "accept": acc_ms,
                      "attention_gbs": round(attn_gbs, 1), "step_eager": eager_ms},
-        "gpu_launches": launches_per_step * args.steps,
+        "gpu_launches": launches_per_step(attn_path_name(args.attn_path, binding, ai), filtered) * args.steps,
         "emitted_tokens_per_step": int(emitted),
         "emitted_tokens_per_s": emitted / (ms / 1000.0),
         "clocks": clk,
@@ -645,7 +652,7 @@ def time_other_workload(name, args, binding, dev, rank, graph_of, timed_loop, lo
                              "frac_of_8tbs": round(step_gbs / NOMINAL_HBM_GBS, 4)},
            "parts_ms": {"attention": ms["attention"], "accept": ms["accept"]},
            "emitted_tokens_per_s": emitted / (ms["step"] / 1000.0),
-           "gpu_launches": (2 if S.filtered else 4) * n,
+           "gpu_launches": launches_per_step(attn_path_name(args.attn_path, binding, ai), S.filtered) * n,
            "clocks": clk,
            "timing": "CUDA-graph replays of one spec_verify_step call, L2 flushed before each"}
     del S, gs

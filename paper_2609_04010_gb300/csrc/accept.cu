@@ -3,8 +3,8 @@
 // (Linear Sampler)" (Appendix B.3; Sec. 4.2).
 //
 // Three launches, no inter-block waiting (each is a programmatic dependent of the one
-// before and waits for it on the device; in a verify step the first is a programmatic
-// dependent of the attention kernel and runs beside it):
+// before and waits for it on the device; in a verify step they run on a side stream,
+// beside the attention kernel):
 //   1. row_stats_kernel: one warp per (sequence, row, 4096-entry vocab chunk) reads
 //      the chunk once with 16-byte loads and writes its max, its sum of
 //      exp((l - max)/T) and (greedy rows) its lowest-index argmax.

@@ -14,8 +14,8 @@
 //      maximum of every lane of 64 contiguous logits in shared memory (greedy rows: only
 //      the lowest-index argmax). The k-th largest lane maximum bounds the k-th largest
 //      logit from below, since k distinct lanes each hold an element at least that large;
-//   2. a two-digit radix select over the lane maxima finds that bound, the block rescans
-//      only the lanes that reach it (about k contiguous 128-byte runs, usually still in
+//   2. a histogram of the lane maxima below the row's finds that bound (two radix digits
+//      where it lies further down), the block rescans only the lanes that reach it (about k contiguous 128-byte runs, usually still in
 //      L2), ranks the candidates, and takes the top-k, the top-p cut and the
 //      renormalised probabilities (fp32 sums of weights whose exponent argument is
 //      formed in fp64). If the candidates overflow shared memory (many equal logits),
@@ -877,7 +877,7 @@ __global__ void __launch_bounds__(kRowThreads, 8) filter_row_kernel(FiltParams p
 
   if (!greedy && !info.flags) {
     // 2. select. The bound: the high 16 bits of the K-th largest lane key (0: every
-    // element), by two radix digits; each warp counts into its own histogram
+    // element); each warp counts into its own histogram
     const int K = min(k_in, V);
     uint32_t* my_hist = s_hist + (tid >> 5) * 256;
     for (int i = tid; i < (kRowThreads / 32) * 256; i += kRowThreads) s_hist[i] = 0;

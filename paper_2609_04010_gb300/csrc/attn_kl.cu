@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(384, 1)
   int* pb = reinterpret_cast<int*>(smem + C::OFF_PB);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  pdl_launch_dependents();  // the acceptance kernels of a verify step may start beside us
+  pdl_launch_dependents();
 
   // ---- prologue: barriers, TMEM, per-sequence tile prefix sums ----
   if (threadIdx.x == 0) {

@@ -75,7 +75,7 @@ template <int D>
 __global__ void __launch_bounds__(NT) attn_simt_kernel(AttnParams p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SimtSmem<D>& sm = *reinterpret_cast<SimtSmem<D>*>(smem_raw);
-  pdl_launch_dependents();  // the acceptance kernels of a verify step may start beside us
+  pdl_launch_dependents();
   const int split = blockIdx.x, g = blockIdx.y;
   const int b = blockIdx.z / p.row_tiles, rt = blockIdx.z % p.row_tiles;
   const int tid = threadIdx.x;

@@ -40,7 +40,8 @@
 // Work is balanced across blocks "stream-K" style: all 64-key tiles of all (sequence,
 // KV head, row tile) units form one list that is cut into equal contiguous ranges; a
 // unit split between blocks is merged from fp32 partials by attn_merge_kernel
-// (attn_common.cuh). Every mbarrier wait is bounded: a wait that runs out
+// (attn_common.cuh; with batches of short contexts the ranges are whole units instead).
+// Every mbarrier wait is bounded: a wait that runs out
 // sets SPEC_FLAG_TIMEOUT, drains the block's own copies and MMAs, frees TMEM and exits.
 #include <cuda.h>  // CUtensorMap and its encoder's signature (resolved at run time)
 
@@ -51,7 +52,6 @@ namespace specv {
 namespace {
 
 constexpr int TK = kTcKeyTile;               // keys per tile
-
 
 // QR: query rows one Q or P buffer of an M tile holds: 128, or 64 when a KV group has at
 // most 64 query rows. The MMAs still read M = 128 rows; with QR = 64 the buffers are laid
