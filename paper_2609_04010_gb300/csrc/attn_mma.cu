@@ -327,7 +327,11 @@ __global__ void __launch_bounds__(MmaCfg<D, HB, MTW>::THREADS, 1)
                 if (!v1) sc[n][t][2 + e] = -INFINITY;
               }
         }
-        // ---- online softmax, the maximum raised only when it grows by more than 2^8 ----
+        // ---- online softmax. The maximum is raised whenever a row's grows: a row's largest
+        // probability is then 1, which bf16 holds exactly. (Raised only past 2^8, as where the
+        // output has to be fetched from tensor memory: the error of 4 rows over 512 keys is
+        // 2.15e-3 instead of 2.00e-3, of 32 rows over 4,096 keys 2.29e-3 instead of 2.07e-3,
+        // and the times are within 0.7%.) ----
         float x0 = -INFINITY, x1 = -INFINITY;
 #pragma unroll
         for (int n = 0; n < NS; ++n)
@@ -340,7 +344,7 @@ __global__ void __launch_bounds__(MmaCfg<D, HB, MTW>::THREADS, 1)
         x1 = fmaxf(x1, __shfl_xor_sync(0xffffffffu, x1, 1));
         x0 = fmaxf(x0, __shfl_xor_sync(0xffffffffu, x0, 2)) * p.scale_log2;
         x1 = fmaxf(x1, __shfl_xor_sync(0xffffffffu, x1, 2)) * p.scale_log2;
-        if (__any_sync(0xffffffffu, x0 > m0 + 8.f || x1 > m1 + 8.f)) {
+        if (__any_sync(0xffffffffu, x0 > m0 || x1 > m1)) {
           const float n0 = fmaxf(m0, x0), n1 = fmaxf(m1, x1);
           const float a0 = m0 == -INFINITY ? 0.f : ex2(m0 - n0), a1 = m1 == -INFINITY ? 0.f : ex2(m1 - n1);
           m0 = n0;
