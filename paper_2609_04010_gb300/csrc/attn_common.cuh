@@ -297,7 +297,7 @@ __device__ __forceinline__ int range_count(int64_t total, const AttnParams& p) {
 }
 
 // Block cta's range [t0, t1) of the virtual tiles (empty past the last range). Equal ranges,
-// or with whole_units (the small-group kernel) equal numbers of units: where no unit can be
+// or with whole_units equal numbers of units: where no unit can be
 // longer than kWholeTiles, one block's turn at a unit costs less than the merge kernel behind
 // the call (10 requests of 216 keys: 15.5 us split, 12.3 whole; 128 of up to 100: 38 and 18.6).
 __device__ __forceinline__ void block_range(const AttnParams& p, const int* pb, int cta, int64_t total, int ctas,

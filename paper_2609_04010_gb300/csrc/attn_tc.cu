@@ -40,9 +40,7 @@
 // Work is balanced across blocks "stream-K" style: all 64-key tiles of all (sequence,
 // KV head, row tile) units form one list that is cut into equal contiguous ranges; a
 // unit split between blocks is merged from fp32 partials by attn_merge_kernel
-// (attn_common.cuh). Units of a few tiles are split too: each part's probabilities are
-// rounded relative to its own maximum (300 keys, 64 rows: a relative error of 2.09e-3, and
-// 2.29e-3 in one piece). Every mbarrier wait is bounded: a wait that runs out sets
+// (attn_common.cuh). Every mbarrier wait is bounded: a wait that runs out sets
 // SPEC_FLAG_TIMEOUT, drains the block's own copies and MMAs, frees TMEM and exits.
 #include <cuda.h>  // CUtensorMap and its encoder's signature (resolved at run time)
 
@@ -625,7 +623,7 @@ __global__ void __launch_bounds__(TcCfg<D, MT, QR, HP>::THREADS, 1)
           for (int c = 0; c < o; ++c) mx[c] = fmaxf(mx[c], mx[c + o]);
         const float tmax = mx[0] * p.scale_log2;  // base 2
         const float m_new = fmaxf(m, tmax);
-        const bool want = k > 0 && m_new > m + 8.f;
+        const bool want = k > 0 && m_new > m + (p.whole_units ? 0.f : 8.f);  // few tiles: the exact maximum
         const bool rescale = __any_sync(0xffffffffu, want);
         float alpha = 1.f;
         if (k == 0) {
@@ -804,6 +802,20 @@ cudaError_t launch_typed(const spec_attn_args_t& a, const AttnPlan& P, char* ws,
   // move real tiles away from blocks that pay no boundary.
   const int64_t units = static_cast<int64_t>(a.batch) * p.hunits * P.row_tiles;
   p.unit_overhead = units > P.grid ? Cf::UNIT_OVERHEAD : 0;
+  // Fewer units than blocks: k whole blocks for each unit rather than a range for every block
+  // where that lengthens the longest range by less than what ranges across two units pay for
+  // the second one (with T tiles in a unit, T / k against T units / grid): 64 units of 1,000
+  // keys and 256 rows 40.8 us in 152 ranges, 36.9 in 128.
+  const int64_t k = P.grid / units, tiles = (p.max_keys + TK - 1) / TK;
+  if (k > 0 && tiles * (P.grid - k * units) < 2 * Cf::UNIT_OVERHEAD * P.grid * k) p.grid = static_cast<int>(k * units);
+  // Short units that would be split in two at most are not split: 64 ragged units of up to
+  // 440 keys and 160 rows take 16.4 us whole, 28 split and merged. With fewer units, splitting
+  // them is as fast and more exact (each part's probabilities are rounded against its own
+  // maximum; 64 rows over 300 keys: a relative error of 2.09e-3 in parts, 2.16e-3 whole).
+  if (k <= 2 && tiles <= kWholeTiles) {
+    p.grid = P.grid;
+    p.whole_units = 1;
+  }
   p.unit_heads = HP;
   if (!p.q_tma) mq = mk;  // unused
   const size_t smem = Cf::smem_bytes(a.batch);
