@@ -207,6 +207,25 @@ def test_small_groups(oracle_mod, case):
     compare_attention(g_out, g_lse, o_out, o_lse)
 
 
+# The row-tile kernel's ranges: short units kept whole (one and two M tiles, head pairs, more
+# units than blocks), and whole blocks for each of fewer units.
+RANGES = [
+    dict(batch=8, gamma=32, num_q_heads=40, num_kv_heads=8, head_dim=64, page_size=16, ctx=(200, 440)),
+    dict(batch=25, gamma=16, num_q_heads=32, num_kv_heads=8, head_dim=128, page_size=16, ctx=(0, 300)),
+    dict(batch=90, gamma=10, num_q_heads=10, num_kv_heads=2, head_dim=128, page_size=32, ctx=(1, 200)),
+    dict(batch=5, gamma=32, num_q_heads=20, num_kv_heads=4, head_dim=128, page_size=16, ctx=1000),
+]
+
+
+@pytest.mark.parametrize("case", range(len(RANGES)))
+def test_row_tile_ranges(oracle_mod, case):
+    inp = W.make_attn_inputs(seed=260 + case, **RANGES[case])
+    g_out, g_lse = gpu_attention(inp, binding.ATTN_AUTO)
+    o_out, o_lse, st = oracle_attn(oracle_mod, inp)
+    assert np.all(st == 0)
+    compare_attention(g_out, g_lse, o_out, o_lse)
+
+
 @pytest.mark.parametrize("case", [0, 2, 3, 6, 9])
 def test_small_groups_tree_mask(oracle_mod, case):
     inp = W.make_attn_inputs(seed=230 + case, **GROUPS[case])
