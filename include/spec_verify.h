@@ -540,14 +540,17 @@ spec_status_t spec_accept_block_noalloc(const spec_accept_args_t* accept, spec_s
  * bounded (about 1 s of SM clock); one that runs out sets SPEC_FLAG_TIMEOUT, the block
  * releases its resources and returns, and the context stays usable. These two calls make
  * that happen on purpose, so that it can be tested: each is the launch of its product
- * call (spec_verify_attention on the tensor-core row-tile path, spec_lm_head_stats), with
+ * call (spec_verify_attention on the tensor-core kernel that SPEC_ATTN_AUTO takes for the
+ * shape, or with any other path on the row-tile kernel; spec_lm_head_stats), with
  * the same arguments, workspace rules and errors, except that the kernel's copy producer
  * issues nothing, so every consumer's wait runs out (about 1 s). Afterwards the workspace
  * status word holds SPEC_FLAG_TIMEOUT (spec_read_device_status returns
- * SPEC_ERR_TIMEOUT and clears it), the outputs are undefined, and the workspace's
- * counters are still zero, so the same workspace serves the next product call.
- * spec_test_attention_wait_timeout returns SPEC_ERR_UNSUPPORTED for shapes the
- * tensor-core row-tile kernel does not take. Nothing traps, faults or waits without bound.
+ * SPEC_ERR_TIMEOUT and clears it) and the workspace's counters are still zero, so the same
+ * workspace serves the next product call. An attention output row that no block finished is
+ * left as it was, or zero with a log-sum-exp of -inf where its unit was split between
+ * blocks; the LM head's outputs are undefined.
+ * spec_test_attention_wait_timeout returns SPEC_ERR_UNSUPPORTED for shapes those
+ * kernels do not take. Nothing traps, faults or waits without bound.
  * ------------------------------------------------------------------------------------- */
 spec_status_t spec_test_attention_wait_timeout(const spec_attn_args_t* attn, void* ws,
                                                size_t ws_bytes, spec_stream_t stream);

@@ -283,9 +283,9 @@ def verify_attention_args(attn: AttnArgs, ws: torch.Tensor, stream=None):
 
 
 def test_attention_wait_timeout_args(attn: AttnArgs, ws: torch.Tensor, stream=None):
-    """Test hook: spec_verify_attention on the tensor-core row-tile path with its copy
-    producers idle, so that the kernel's bounded waits run out (about 1 s) and it returns
-    with SPEC_FLAG_TIMEOUT set."""
+    """Test hook: spec_verify_attention on the tensor-core kernel that ATTN_AUTO takes (with
+    any other path: the row-tile kernel), its copy producers idle, so that the kernel's
+    bounded waits run out (about 1 s) and it returns with SPEC_FLAG_TIMEOUT set."""
     _raise(lib().spec_test_attention_wait_timeout(ctypes.byref(attn), _ptr(ws), ws.numel(),
                                                   _stream(stream)), "spec_test_attention_wait_timeout")
 

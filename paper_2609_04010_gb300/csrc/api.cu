@@ -519,11 +519,13 @@ spec_status_t spec_test_attention_wait_timeout(const spec_attn_args_t* attn, voi
   size_t attn_base = 0;
   if (required_bytes(attn, nullptr, nullptr, scope.sms, &attn_base) > ws_bytes)
     return SPEC_ERR_WORKSPACE_TOO_SMALL;
-  const AttnPlan P = attn_plan(*attn, attn_base, scope.sms, SPEC_ATTN_TENSOR_CORES);
+  const AttnPlan P = attn_plan(*attn, attn_base, scope.sms,
+                               attn->path == SPEC_ATTN_AUTO ? SPEC_ATTN_AUTO : SPEC_ATTN_TENSOR_CORES);
   if (P.path != SPEC_ATTN_TENSOR_CORES || P.keys_on_lanes) return SPEC_ERR_UNSUPPORTED;
-  return launch_attn_tc(*attn, P, static_cast<char*>(ws), stream, /*starve=*/true) == cudaSuccess
-             ? SPEC_OK
-             : SPEC_ERR_CUDA;
+  const cudaError_t e = P.heads > 0
+                            ? launch_attn_mma(*attn, P, static_cast<char*>(ws), stream, /*starve=*/true)
+                            : launch_attn_tc(*attn, P, static_cast<char*>(ws), stream, /*starve=*/true);
+  return e == cudaSuccess ? SPEC_OK : SPEC_ERR_CUDA;
 }
 
 spec_status_t spec_verify_step(const spec_attn_args_t* attn, const spec_accept_args_t* accept,

@@ -340,6 +340,24 @@ __device__ __forceinline__ void note_split(const AttnParams& p, int cta, const S
   p.splits[cta] = d;
 }
 
+// A block whose waits ran out leaves units without their partials: the slots of its range's
+// first and last units (no other can be split) are marked bad, as a malformed sequence's are,
+// so that those units' outputs become zeros instead of what an earlier call left in the slots.
+// (Every thread; the range is worked out again, so that the roles need not keep it.)
+template <int TK>
+__device__ __forceinline__ void drop_partials(const AttnParams& p, const int* pb) {
+  const int64_t total = pb[p.batch];
+  int64_t t0, t1;
+  block_range(p, pb, blockIdx.x, total, range_count(total, p), t0, t1);
+  if (t1 <= t0) return;
+#pragma unroll 1
+  for (int i = 0; i < 2; ++i) {
+    const int64_t slot = locate<TK>(i == 0 ? t0 : t1 - 1, t1, p, pb, p.unit_overhead).u + blockIdx.x;
+    for (int r = threadIdx.x; r < p.slot_rows; r += blockDim.x)
+      p.partial_ml[slot * p.slot_rows + r] = make_float2(-INFINITY, -1.f);
+  }
+}
+
 // RW rows of one warp from their partial slots [slot0, slot0 + nsl), SB slots at a time: the
 // loads of all those rows and slots are in flight together.
 template <int D, int RW, int SB>

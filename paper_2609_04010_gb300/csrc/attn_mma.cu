@@ -168,10 +168,10 @@ __global__ void __launch_bounds__(MmaCfg<D, HB, MTW>::THREADS, 1)
     const uint32_t ring = sbase + (warp == 0 ? 0u : C::OFF_V);
     const uint32_t box_bytes = static_cast<uint32_t>(box_keys) * D * 2 * HB;
     const Seg s_first = locate<KS>(t0, t1, p, pb, OVH);
-    for (Seg s = s_first; s.ntile > 0 && ok;) {
+    for (Seg s = s_first; s.ntile > 0 && ok && !p.starve;) {
       for (int k = 0; k < s.ntile; ++k, ++it) {
         const uint32_t st = it % S;
-        if (it >= S) ok = mbar_wait(empty(st), ((it / S) - 1) & 1, abort_flag, p.status);
+        if (it >= S) ok = mbar_wait_warp(empty(st), ((it / S) - 1) & 1, abort_flag, p.status);
         if (!ok) break;
         const int key0 = (s.tile0 + k) * KS;
         // boxes with a visible key; a malformed sequence reads nothing
@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(MmaCfg<D, HB, MTW>::THREADS, 1)
       for (int k = 0; k < s.ntile; ++k, ++it) {
         if (C::KG > 1 && it % C::KG != static_cast<uint32_t>(kg)) continue;
         const uint32_t st = it % S;
-        ok = __all_sync(0xffffffffu, mbar_wait(full(st), (it / S) & 1, abort_flag, p.status));
+        ok = mbar_wait_warp(full(st), (it / S) & 1, abort_flag, p.status);
         if (!ok) break;
         bad |= stage_bad[st] != 0;
         const int key0 = (s.tile0 + k) * KS;
@@ -425,7 +425,7 @@ __global__ void __launch_bounds__(MmaCfg<D, HB, MTW>::THREADS, 1)
         float* xch = reinterpret_cast<float*>(smem + C::OFF_XCH);
         if (kg > 0) {
           if (seg_no > 0)
-            ok = __all_sync(0xffffffffu, mbar_wait(xch_free(pair), (seg_no - 1) & 1, abort_flag, p.status));
+            ok = mbar_wait_warp(xch_free(pair), (seg_no - 1) & 1, abort_flag, p.status);
           if (!ok) break;
           float* mine = xch + ((kg - 1) * C::PAIRS + pair) * (C::XCH_WARP / 4) + lane;
 #pragma unroll
@@ -442,7 +442,7 @@ __global__ void __launch_bounds__(MmaCfg<D, HB, MTW>::THREADS, 1)
           s = locate<KS>(s.vnext, t1, p, pb, OVH);
           continue;
         }
-        ok = __all_sync(0xffffffffu, mbar_wait(xch_full(pair), seg_no & 1, abort_flag, p.status));
+        ok = mbar_wait_warp(xch_full(pair), seg_no & 1, abort_flag, p.status);
         if (!ok) break;
 #pragma unroll 1
         for (int g = 0; g < C::KG - 1; ++g) {
@@ -509,6 +509,8 @@ __global__ void __launch_bounds__(MmaCfg<D, HB, MTW>::THREADS, 1)
       s = locate<KS>(s.vnext, t1, p, pb, OVH);
     }
   }
+  __syncthreads();
+  if (*abort_flag) drop_partials<KS>(p, pb);
 }
 
 // ---------------------------------------------------------------------------------
@@ -539,7 +541,8 @@ int shift_of(int x) {
 }
 
 template <int D, int HB, int MTW>
-cudaError_t launch_typed(const spec_attn_args_t& a, const AttnPlan& P, char* ws, cudaStream_t stream) {
+cudaError_t launch_typed(const spec_attn_args_t& a, const AttnPlan& P, char* ws, cudaStream_t stream,
+                         bool starve) {
   using C = MmaCfg<D, HB, MTW>;
   const int box_keys = std::min(a.page_size, C::KS);
   CUtensorMap mk, mv;
@@ -553,6 +556,7 @@ cudaError_t launch_typed(const spec_attn_args_t& a, const AttnPlan& P, char* ws,
   p.grid = P.grid;
   p.min_tiles = kMmaMinTiles;
   p.unit_heads = HB;
+  p.starve = starve ? 1 : 0;
   p.whole_units = p.max_keys <= kWholeTiles * C::KS ? 1 : 0;
   const size_t smem = C::smem_bytes(a.batch);
   auto kernel = attn_mma_kernel<D, HB, MTW>;
@@ -565,9 +569,10 @@ cudaError_t launch_typed(const spec_attn_args_t& a, const AttnPlan& P, char* ws,
 }
 
 template <int D, int HB>
-cudaError_t launch_rows(const spec_attn_args_t& a, const AttnPlan& P, char* ws, cudaStream_t stream) {
-  if (P.rows <= 16) return launch_typed<D, HB, 1>(a, P, ws, stream);
-  if constexpr (HB <= 4) return launch_typed<D, HB, 2>(a, P, ws, stream);
+cudaError_t launch_rows(const spec_attn_args_t& a, const AttnPlan& P, char* ws, cudaStream_t stream,
+                        bool starve) {
+  if (P.rows <= 16) return launch_typed<D, HB, 1>(a, P, ws, stream, starve);
+  if constexpr (HB <= 4) return launch_typed<D, HB, 2>(a, P, ws, stream, starve);
   return cudaErrorInvalidValue;  // not planned (mma_heads)
 }
 
@@ -583,12 +588,14 @@ int mma_heads(const spec_attn_args_t& a, int rows) {
   return 2;
 }
 
-cudaError_t launch_attn_mma(const spec_attn_args_t& a, const AttnPlan& P, char* ws, cudaStream_t stream) {
+cudaError_t launch_attn_mma(const spec_attn_args_t& a, const AttnPlan& P, char* ws, cudaStream_t stream,
+                            bool starve) {
   if (a.head_dim == 128)
-    return P.heads == 4 ? launch_rows<128, 4>(a, P, ws, stream) : launch_rows<128, 2>(a, P, ws, stream);
-  return P.heads == 8   ? launch_rows<64, 8>(a, P, ws, stream)
-         : P.heads == 4 ? launch_rows<64, 4>(a, P, ws, stream)
-                        : launch_rows<64, 2>(a, P, ws, stream);
+    return P.heads == 4 ? launch_rows<128, 4>(a, P, ws, stream, starve)
+                        : launch_rows<128, 2>(a, P, ws, stream, starve);
+  return P.heads == 8   ? launch_rows<64, 8>(a, P, ws, stream, starve)
+         : P.heads == 4 ? launch_rows<64, 4>(a, P, ws, stream, starve)
+                        : launch_rows<64, 2>(a, P, ws, stream, starve);
 }
 
 }  // namespace specv

@@ -778,6 +778,7 @@ __global__ void __launch_bounds__(TcCfg<D, MT, QR, HP>::THREADS, 1)
     tc_fence_before();
   }
   __syncthreads();
+  if (*abort_flag) drop_partials<TK>(p, pb);
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, C::TMEM_COLS);

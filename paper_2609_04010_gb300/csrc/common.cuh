@@ -182,7 +182,7 @@ cudaError_t launch_attn_simt(const spec_attn_args_t& a, const AttnPlan& P, char*
 cudaError_t launch_attn_tc(const spec_attn_args_t& a, const AttnPlan& P, char* ws,
                            cudaStream_t stream, bool starve = false);
 cudaError_t launch_attn_mma(const spec_attn_args_t& a, const AttnPlan& P, char* ws,
-                            cudaStream_t stream);
+                            cudaStream_t stream, bool starve = false);
 // KV heads one block of the small-group kernel serves (2, 4 or 8), or 0 where it does not
 // apply: more than kMmaMaxRows query rows per KV head, an odd Hkv, or a batch whose prefix
 // sums do not fit beside its stages.

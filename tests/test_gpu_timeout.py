@@ -86,3 +86,43 @@ def test_lm_head_wait_runs_out(oracle_mod):
     Te = np.array([float(T[r // rps]) if T[r // rps] > 0 else 1.0 for r in range(R)])
     np.testing.assert_array_less(np.abs(out["row_sum"].cpu().numpy() - o["row_sum"]),
                                  o["row_sum"] * (1e-4 + 2 * err / Te))
+
+
+# (group, gamma, hkv, head dim, path): the small-group kernel with one, two and four key
+# groups at head dim 128 and one at 64, then the row-tile kernel's three forms
+STALE = [(4, 8, 4, 128, "auto"), (4, 4, 4, 128, "auto"), (4, 1, 2, 128, "auto"), (2, 8, 8, 64, "auto"),
+         (4, 8, 2, 128, "tc"), (4, 16, 2, 128, "tc"), (8, 32, 2, 128, "tc")]
+
+
+@pytest.mark.parametrize("group,gamma,hkv,dim,path", STALE)
+def test_attention_timeout_leaves_no_stale_output(oracle_mod, group, gamma, hkv, dim, path):
+    # A call that timed out returns nothing that an earlier call on the workspace left in the
+    # partials: a row is untouched, or zero with a log-sum-exp of -inf (a split unit). The
+    # contexts are long enough for units to be split.
+    inp = W.make_attn_inputs(3, gamma, group * hkv, hkv, dim, 16, (900, 2500), True, seed=191 + gamma)
+    q, k, v, pt, kl = attn_tensors(inp)
+    out = torch.empty_like(q)
+    lse = torch.empty(q.shape[:3], dtype=torch.float32, device=q.device)
+    a = binding.attn_args(q, k, v, pt, kl, out, lse,
+                          path=binding.ATTN_AUTO if path == "auto" else binding.ATTN_TENSOR_CORES)
+    ws = binding.new_workspace(binding.workspace_size(a, None))
+    o_out, o_lse, st = oracle_mod.verify_attention(inp.q, inp.k_cache, inp.v_cache, inp.page_table,
+                                                   inp.kv_len, gamma)
+    assert np.all(st == 0)
+    for _ in range(2):
+        binding.verify_attention_args(a, ws)  # its partials stay in the workspace
+        torch.cuda.synchronize()
+        assert read_status(ws) == (0, 0)
+        compare_attention(out.float().cpu().numpy(), lse.cpu().numpy(), o_out, o_lse)
+        out.fill_(7.0)
+        lse.fill_(7.0)
+        binding.test_attention_wait_timeout_args(a, ws)
+        torch.cuda.synchronize()
+        code, flags = read_status(ws)
+        assert code == SPEC_ERR_TIMEOUT and flags & binding.FLAG_TIMEOUT, (code, flags)
+        assert read_status(ws) == (0, 0)
+        rows, ends = out.float(), lse
+        dropped = torch.isneginf(ends)
+        assert bool(dropped.any())  # some unit was split
+        assert bool((dropped | (ends == 7.0)).all()), "a log-sum-exp of an earlier call"
+        assert bool((rows == torch.where(dropped, 0.0, 7.0)[..., None]).all()), "an output of an earlier call"
