@@ -52,7 +52,7 @@ FilterLayout filter_layout(const spec_accept_args_t& a, int max_top_k, size_t ba
   L.lanes_per_split = static_cast<int>((L.nlanes + splits - 1) / splits);
   L.splits = (L.nlanes + L.lanes_per_split - 1) / L.lanes_per_split;
   L.cand_cap = 512;
-  while (L.cand_cap < 4 * max_top_k && L.cand_cap < 2048) L.cand_cap <<= 1;
+  while (L.cand_cap < 4 * max_top_k && L.cand_cap < kFiltMaxCand) L.cand_cap <<= 1;
   // region A holds the lane maxima, then the ranked candidates (8 B each), then the
   // draw's four lists, each padded to a power of two for the bitonic sort
   int mk2 = 1;
@@ -75,6 +75,9 @@ namespace {
 
 constexpr int kRowUnroll = 8;        // 16-byte loads in flight per thread
 constexpr int kStageGranules = 4 * kRowThreads;  // 16-byte granules of an unaligned row staged at a time
+// dynamic shared memory of a block at most: lane maxima or sorted lists, candidates, the stage
+constexpr size_t kMaxSmem = (kFiltMaxLanes * 4 > kFilterMaxTopK * 16 ? kFiltMaxLanes * 4 : kFilterMaxTopK * 16) +
+                            kFiltMaxCand * 12 + (kStageGranules + 1) * 16;
 constexpr int kRankSortMax = 256;    // candidates ranked by counting; more are sorted bitonically
 constexpr uint32_t kRowBadLogits = 1u, kRowBadFilter = 2u;
 
@@ -1165,8 +1168,7 @@ cudaError_t launch_filtered_typed(const FiltParams& p, cudaStream_t stream, bool
   cfg.numAttrs = overlap_prior ? 1 : 0;  // beside the attention kernel of a verify step
   cudaError_t e = cudaSuccess;
   if (!VEC)  // the stage may take a block past 48 KB
-    e = cudaFuncSetAttribute(filter_row_kernel<BF16, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(cfg.dynamicSmemBytes));
+    e = allow_smem(filter_row_kernel<BF16, VEC>, kMaxSmem);
   if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, filter_row_kernel<BF16, VEC>, p);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();

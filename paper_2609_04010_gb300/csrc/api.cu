@@ -163,8 +163,6 @@ spec_accept_args_t draft_as_accept(const spec_draft_args_t& d) {
   return a;
 }
 
-constexpr size_t kDraftMaxSmem = 200 * 1024;  // lane summaries of one unfiltered draw block
-
 size_t draft_bytes(const spec_draft_args_t& d, const spec_filter_args_t* f, int sms, bool vec) {
   if (f) return filter_layout(draft_as_accept(d), f->max_top_k, kWsHeader, sms, true).end;
   return draft_layout(d, kWsHeader, sms, vec).end;

@@ -660,8 +660,7 @@ cudaError_t launch_rh(const spec_attn_args_t& a, const AttnPlan& P, char* ws, cu
   p.unit_overhead = units > P.grid ? Cf::UNIT_OVERHEAD : 0;
   const size_t smem = Cf::smem_bytes(a.batch);
   auto kernel = attn_kl_kernel<RH>;
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+  cudaError_t e = allow_smem(kernel, kTcMaxSmem);
   if (e != cudaSuccess) return e;
   kernel<<<P.grid, Cf::THREADS, smem, stream>>>(mk, mv, mq, p);
   return cudaGetLastError();

@@ -560,8 +560,7 @@ cudaError_t launch_typed(const spec_attn_args_t& a, const AttnPlan& P, char* ws,
   p.whole_units = p.max_keys <= kWholeTiles * C::KS ? 1 : 0;
   const size_t smem = C::smem_bytes(a.batch);
   auto kernel = attn_mma_kernel<D, HB, MTW>;
-  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             static_cast<int>(smem));
+  const cudaError_t e = allow_smem(kernel, kTcMaxSmem);
   if (e != cudaSuccess) return e;
   kernel<<<P.grid, C::THREADS, smem, stream>>>(mk, mv, p, shift_of(a.page_size), shift_of(box_keys));
   const cudaError_t launched = cudaGetLastError();

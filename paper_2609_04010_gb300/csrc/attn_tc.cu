@@ -821,8 +821,7 @@ cudaError_t launch_typed(const spec_attn_args_t& a, const AttnPlan& P, char* ws,
   if (!p.q_tma) mq = mk;  // unused
   const size_t smem = Cf::smem_bytes(a.batch);
   auto kernel = a.tree_mask ? attn_tc_kernel<D, MT, true, QR, HP> : attn_tc_kernel<D, MT, false, QR, HP>;
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+  cudaError_t e = allow_smem(kernel, kTcMaxSmem);
   if (e != cudaSuccess) return e;
   kernel<<<P.grid, Cf::THREADS, smem, stream>>>(mk, mv, mq, p);
   e = cudaGetLastError();

@@ -48,6 +48,7 @@ AcceptLayout accept_layout(const spec_accept_args_t& a, size_t base);
 // --- filtered acceptance ---
 constexpr int kFilterMaxTopK = SPEC_FILTER_MAX_TOP_K;
 constexpr int kFiltLaneElems = 64;    // contiguous logits per lane (at the smallest lane size)
+constexpr int kFiltMaxCand = 2048;    // candidates one row block holds at most
 constexpr int kFiltMaxLanes = 4096;   // lane maxima one row block keeps in shared memory
 constexpr int kFiltBlocksPerSm = 8;   // row blocks resident per SM (128 threads each)
 constexpr int kFiltMaxSplits = 16;    // blocks one row may be split across
@@ -81,6 +82,7 @@ FilterLayout filter_layout(const spec_accept_args_t& a, int max_top_k, size_t ba
                            bool draw = false);
 
 // --- draft-side sampling ---
+constexpr size_t kDraftMaxSmem = 200 * 1024;  // lane summaries of one unfiltered draw block
 struct DraftLayout {
   size_t tickets;      // uint32 [batch]: rows of the sequence finished (reset by the last)
   size_t row_flags;    // uint32 [batch][gamma]
@@ -253,6 +255,13 @@ size_t tc_smem_bytes(int head_dim, int rows_per_cta, int rows, int batch, bool h
 bool tc_head_pair(int head_dim, int rows, int num_kv_heads, int batch);
 constexpr int kTcMaxBatch = 4096;  // batch prefix sums live in shared memory
 constexpr size_t kTcMaxSmem = 227u * 1024u;  // dynamic shared memory of one block
+// A kernel's limit of dynamic shared memory belongs to the function, not to a call: it is
+// always set to the most any call can need, so that no host thread lowers it between another
+// thread's setting and its launch.
+template <class Kernel>
+cudaError_t allow_smem(Kernel kernel, size_t most) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most));
+}
 
 }  // namespace specv
 

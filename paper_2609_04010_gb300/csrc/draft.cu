@@ -588,9 +588,8 @@ template <bool BF16, bool VEC>
 cudaError_t launch_draft_typed(const DraftParams& p, size_t smem, cudaStream_t stream) {
   if (!VEC) smem = (smem + 15) / 16 * 16 + (kStageGranules + 1) * 16;  // the stage of unaligned rows
   if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(draft_sample_kernel<BF16, VEC>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               static_cast<int>(smem));
+    const cudaError_t e = allow_smem(draft_sample_kernel<BF16, VEC>,
+                                     kDraftMaxSmem + (VEC ? 0 : (kStageGranules + 1) * 16));
     if (e != cudaSuccess) return e;
   }
   draft_sample_kernel<BF16, VEC><<<dim3(p.splits, p.gamma, p.batch), kThreads, smem, stream>>>(p);
