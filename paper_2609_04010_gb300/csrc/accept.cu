@@ -517,8 +517,10 @@ __global__ void __launch_bounds__(kDecideThreads) decide_kernel(AcceptParams p) 
       qt = 1.f;
     } else {
       const double pd = s_prob[0][i], qd = s_prob[1][i], u = static_cast<double>(my_u);
-      // u > min(1, p / q) as u > 1 or u q > p; q_i(t_i) = 0 (underflow): accept iff p > 0
-      reject = u > 1.0 || (qd > 0.0 ? u * qd > pd : !(pd > 0.0) && u > 0.0);
+      // u > min(1, p / q) as u > 1 or u q > p, both scaled by 2^200: a product of u and a
+      // subnormal q would round to zero or to a neighbour, and a draft that p gives nothing
+      // be taken. q_i(t_i) = 0 (underflow): accept iff p > 0
+      reject = u > 1.0 || (qd > 0.0 ? (u * 0x1p200) * qd > pd * 0x1p200 : !(pd > 0.0) && u > 0.0);
       pt = static_cast<float>(pd);
       qt = static_cast<float>(qd);
     }

@@ -268,3 +268,25 @@ def test_rows_at_every_alignment(oracle_mod, dtype, vocab, shift):
     o = oracle_accept(oracle_mod, inp)
     ties = compare_accept({k: v.cpu().numpy() for k, v in r.items()}, o, inp.gamma)
     assert len(ties) <= 1, ties
+
+
+@pytest.mark.parametrize("p_logit,q_logit", [(-np.inf, -744.5), (-np.inf, -743.75), (-744.5, -743.75)])
+@pytest.mark.parametrize("u", [2.0 ** -24, 0.125, 0.25, 0.375, 0.625, 1.0])
+def test_subnormal_draft_probabilities(oracle_mod, p_logit, q_logit, u):
+    # q_i(t_i) is one or two units of the smallest subnormal number and p_i(t_i) is zero or one
+    # of them: u q_i(t_i) is not to be rounded there (p = 0 rejects for every u > 0, p / q = 1/2
+    # for u > 1/2)
+    V, gamma = 40, 3
+    inp = W.make_accept_inputs(1, gamma, V, "f32", 1.0, 1.0, [1.0], seed=8)
+    target, drafter, tokens = inp.target_logits, inp.drafter_logits, inp.block_tokens
+    target[:], drafter[:] = -np.inf, -np.inf
+    target[..., 3], drafter[..., 0] = 0.0, 0.0  # p and q on different tokens but for the draft
+    tokens[:], tokens[0, 1] = 0, 7
+    target[0, 0, 7], drafter[0, 1, 7] = p_logit, q_logit
+    inp.uniforms[:] = 0.5
+    inp.uniforms[0, 0] = u
+    g, o = gpu_accept(inp), oracle_accept(oracle_mod, inp)
+    reject = u > (0.0 if np.isinf(p_logit) else 0.5)
+    assert bool(o["num_accepted"][0] == 0) == reject and o["status"][0] == 0
+    assert g["num_accepted"][0] == o["num_accepted"][0]
+    np.testing.assert_array_equal(g["out_tokens"][0], o["out_tokens"][0])
