@@ -361,11 +361,23 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
   return r;
 }
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
 __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   uint64_t r;
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
+
+// The weight 2^((x - m) c) may be taken as 2^(x c - m c), one multiply-add with m c rounded,
+// while |m c| <= kFusedMax: the rounding, at most 2^-19, is 1.3e-6 of every weight. Beyond it
+// (large logits, low temperatures) it grows with m c, to factors of 2 at 2^24 and to overflow,
+// and the difference is formed first.
+constexpr float kFusedMax = 64.f;
+__device__ __forceinline__ bool past_fused(float m, float c) { return fabsf(m * c) > kFusedMax && m > -INFINITY; }
 
 // Programmatic dependent launch: let the next kernel on the stream start now / wait for
 // the kernel this one depends on (no-ops for kernels launched without the attribute).

@@ -20,6 +20,7 @@
 #include <cfloat>
 #include <climits>
 #include <cmath>
+#include <type_traits>
 
 #include "common.cuh"
 
@@ -151,7 +152,7 @@ __device__ __forceinline__ void gather8(float r, int i, float* v) {
 // lane, but for the 8 lanes together: each exchange halves the lanes a thread still
 // carries, 7 shuffles for 8 maxima (two bf16 to a word) and 7 for 8 sums instead of 24
 // each, and thread i of a group ends with lane k = i. 1,024 rows of 128,256 logits: 72.4 us
-// with butterflies and one shared atomic per lane in the pick below, now 54.5 (4.82 TB/s).
+// with butterflies and one shared atomic per lane in the pick below, now 53.4 (4.92 TB/s).
 __device__ __forceinline__ void scan_bf16(const uint4* dv, int v0, int vend, int l0, int n,
                                           float c, bool greedy, float2* lanes, float& m, int& a, uint32_t& nacc,
                                           bool& bad) {
@@ -204,30 +205,37 @@ __device__ __forceinline__ void scan_bf16(const uint4* dv, int v0, int vend, int
   w[1] = b0 ? r0 : o0;
   w[2] = b0 ? o1 : r1;
   w[3] = b0 ? r1 : o1;
+  // The lanes' weights 2^((x - lm) c), by one multiply-add each unless one of the warp's lanes
+  // is past that (one vote for 8 vectors; a test for each took 54.9 us instead of 53.4). A NaN
+  // logit makes its lane's sum NaN (tested once per lane below), except in a lane with no
+  // finite maximum, whose words are tested here.
   float ls[8];
+  auto sums = [&](auto fused) {
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const float lm = k < 4 ? lo_f(w[k & 3]) : hi_f(w[k & 3]);
-    const uint32_t wv[4] = {dv[k].x, dv[k].y, dv[k].z, dv[k].w};
-    // The lane's weights 2^((x - lm) c), each argument one multiply-add. A NaN logit makes its
-    // lane's sum NaN (tested once per lane below), except in a lane with no finite maximum,
-    // whose words are tested here.
-    const float nlc = -lm * c;
-    float sum = 0.f;
+    for (int k = 0; k < 8; ++k) {
+      const float lm = k < 4 ? lo_f(w[k & 3]) : hi_f(w[k & 3]);
+      const uint32_t wv[4] = {dv[k].x, dv[k].y, dv[k].z, dv[k].w};
+      const float nlc = -lm * c;
+      float sum = 0.f;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      float e0, e1;
-      unpack2(fma2(pack2(lo_f(wv[q]), hi_f(wv[q])), pack2(c, c), pack2(nlc, nlc)), e0, e1);
-      sum += ex2(e0);
-      sum += ex2(e1);
+      for (int q = 0; q < 4; ++q) {
+        const uint64_t x = pack2(lo_f(wv[q]), hi_f(wv[q]));
+        float e0, e1;
+        unpack2(decltype(fused)::value ? fma2(x, pack2(c, c), pack2(nlc, nlc))
+                                       : mul2(add2(x, pack2(-lm, -lm)), pack2(c, c)), e0, e1);
+        sum += ex2(e0);
+        sum += ex2(e1);
+      }
+      if (lm == -INFINITY) {
+        sum = 0.f;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) nacc |= (wv[q] & 0x7FFF7FFFu) + 0x007F007Fu;
+      }
+      ls[k] = sum;
     }
-    if (lm == -INFINITY) {
-      sum = 0.f;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) nacc |= (wv[q] & 0x7FFF7FFFu) + 0x007F007Fu;
-    }
-    ls[k] = sum;
-  }
+  };
+  if (__any_sync(0xffffffffu, past_fused(b2 ? hi_f(kk) : lo_f(kk), c))) sums(std::false_type{});
+  else sums(std::true_type{});
   const float s = reduce8<8>(ls, i, [](float x, float y) { return x + y; });
   const int vi = v0 + i * kThreads + (tid & ~7);  // the first vector of lane k = i
   if (vi < vend) {
@@ -310,20 +318,26 @@ __global__ void __launch_bounds__(kThreads, 8) draft_sample_kernel(DraftParams p
         const float mine = reduce8<kGroup>(lm, i, [](float x, float y) { return fmaxf(x, y); });
         gather8(mine, i, lm);
         float ls[kUnroll];
+        auto sums = [&](auto fused) {  // (as in scan_bf16)
 #pragma unroll
-        for (int k = 0; k < kUnroll; ++k) {
-          const uint32_t wv[4] = {dv[k].x, dv[k].y, dv[k].z, dv[k].w};
-          // (as in scan_bf16)
-          ls[k] = 0.f;
-          if (lm[k] != -INFINITY) {
-            const float nlc = -lm[k] * c;
+          for (int k = 0; k < kUnroll; ++k) {
+            const uint32_t wv[4] = {dv[k].x, dv[k].y, dv[k].z, dv[k].w};
+            ls[k] = 0.f;
+            if (lm[k] != -INFINITY) {
+              const float nlc = -lm[k] * c;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) ls[k] += ex2(fmaf(__uint_as_float(wv[q]), c, nlc));
-          } else {
+              for (int q = 0; q < 4; ++q) {
+                const float x = __uint_as_float(wv[q]);
+                ls[k] += ex2(decltype(fused)::value ? fmaf(x, c, nlc) : (x - lm[k]) * c);
+              }
+            } else {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) nacc |= (wv[q] & nan_mask) + nan_add;
+              for (int q = 0; q < 4; ++q) nacc |= (wv[q] & nan_mask) + nan_add;
+            }
           }
-        }
+        };
+        if (__any_sync(0xffffffffu, past_fused(mine, c))) sums(std::false_type{});
+        else sums(std::true_type{});
         const float sum = reduce8<kGroup>(ls, i, [](float x, float y) { return x + y; });
         const int vi = v0 + i * kThreads + (tid & ~(kGroup - 1));  // the first vector of lane i
         if ((tid & 8) == 0 && vi < vend) {
@@ -545,7 +559,7 @@ __global__ void __launch_bounds__(kThreads, 8) draft_sample_kernel(DraftParams p
       }
       if (tid == 0) {
         s_tok = t;
-        s_q = wt / S;
+        s_q = fminf(wt / S, 1.f);  // S may be rounded below its only weight
       }
     }
     __syncthreads();

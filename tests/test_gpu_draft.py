@@ -219,3 +219,23 @@ def test_sample_rows_at_every_alignment(oracle_mod, dtype, vocab, shift):
     same = g == o["tokens"]
     assert np.all(same | (o["margin"] < TIE_MARGIN))
     np.testing.assert_allclose(q[same], o["q_tok"][same], rtol=DIAG_RTOL)
+
+
+@pytest.mark.parametrize("vocab,dtype", [(4096, "bf16"), (4099, "bf16"), (4096, "f32"), (4099, "f32"), (40000, "bf16")])
+@pytest.mark.parametrize("shift", [20.0, -200.0])
+def test_low_temperatures_and_large_logits(oracle_mod, vocab, dtype, shift):
+    # |max| / T from 200 to 2e10: a weight's exponent (x - max) / T is small where x / T and
+    # max / T are not, and 40 tokens of each row share its maximum
+    temps = [0.1, 1e-2, 1e-3, 1e-6, 1e-8]
+    dl, T, u = draft_inputs(10, 4, vocab, "f32", temps, seed=vocab)
+    rng = np.random.default_rng(vocab)
+    x = dl.astype(np.float32) + np.float32(shift)
+    if dtype == "bf16":  # round to bf16
+        x = torch.from_numpy(x).to(torch.bfloat16).float().numpy()
+    for b in range(x.shape[0]):
+        for j in range(x.shape[1]):
+            x[b, j, rng.choice(vocab, 40, replace=False)] = x[b, j].max()
+    if dtype == "bf16":
+        x = (x.view(np.uint32) >> 16).astype(np.uint16)
+    g, o = check(oracle_mod, x, T, u)
+    assert np.all(o["status"] == 0) and np.all(g["q_tok"] <= 1.0)
