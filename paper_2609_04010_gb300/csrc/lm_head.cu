@@ -22,6 +22,7 @@
 #include <cfloat>
 #include <climits>
 #include <cmath>
+#include <type_traits>
 
 #include "lm_head.cuh"
 #include "tc_ptx.cuh"
@@ -202,7 +203,7 @@ struct RowStats {
 // W logits of this thread's row, at vocabulary indices col0.., of which the first nv are
 // real, folded into its statistics. About 3.5 instructions a logit: a tree of maxima, one
 // packed multiply-add for the non-finite test (x * 0 is NaN for NaN and infinities), one
-// for the exponent's argument, a packed sum. The index of a new maximum and the token's
+// for the exponent's argument (two operations past kFusedMax), a packed sum. The index of a new maximum and the token's
 // logit are looked for only in the columns that hold one. With compare-and-select chains
 // per logit, about 10 instructions in series, the heads above took 177.7 and 716.7 us.
 template <int W>
@@ -237,28 +238,33 @@ __device__ __forceinline__ void reduce_columns(RowStats& st, uint32_t* r, int co
   }
   const float mc = st.m > -INFINITY ? -st.m * st.c2 : 0.f;
   const uint64_t c22 = pack2(st.c2, st.c2), mc2 = pack2(mc, mc), zero = pack2(0.f, 0.f);
+  const uint64_t m2 = pack2(-st.m, -st.m);
   uint64_t s0 = zero, s1 = zero, z0 = zero, z1 = zero;
+  auto sums = [&](auto fused) {
 #pragma unroll
-  for (int e = 0; e < W; e += 4) {
-    const uint64_t v0 = pack2(x[e], x[e + 1]), v1 = pack2(x[e + 2], x[e + 3]);
-    z0 = fma2(v0, zero, z0);
-    z1 = fma2(v1, zero, z1);
-    float a0, a1, a2, a3;
-    unpack2(fma2(v0, c22, mc2), a0, a1);
-    unpack2(fma2(v1, c22, mc2), a2, a3);
-    a0 = ex2(a0);
-    a1 = ex2(a1);
-    a2 = ex2(a2);
-    a3 = ex2(a3);
-    if (nv < W) {
-      a0 = e < nv ? a0 : 0.f;
-      a1 = e + 1 < nv ? a1 : 0.f;
-      a2 = e + 2 < nv ? a2 : 0.f;
-      a3 = e + 3 < nv ? a3 : 0.f;
+    for (int e = 0; e < W; e += 4) {
+      const uint64_t v0 = pack2(x[e], x[e + 1]), v1 = pack2(x[e + 2], x[e + 3]);
+      z0 = fma2(v0, zero, z0);
+      z1 = fma2(v1, zero, z1);
+      float a0, a1, a2, a3;
+      unpack2(decltype(fused)::value ? fma2(v0, c22, mc2) : mul2(add2(v0, m2), c22), a0, a1);
+      unpack2(decltype(fused)::value ? fma2(v1, c22, mc2) : mul2(add2(v1, m2), c22), a2, a3);
+      a0 = ex2(a0);
+      a1 = ex2(a1);
+      a2 = ex2(a2);
+      a3 = ex2(a3);
+      if (nv < W) {
+        a0 = e < nv ? a0 : 0.f;
+        a1 = e + 1 < nv ? a1 : 0.f;
+        a2 = e + 2 < nv ? a2 : 0.f;
+        a3 = e + 3 < nv ? a3 : 0.f;
+      }
+      s0 = add2(s0, pack2(a0, a1));
+      s1 = add2(s1, pack2(a2, a3));
     }
-    s0 = add2(s0, pack2(a0, a1));
-    s1 = add2(s1, pack2(a2, a3));
-  }
+  };
+  if (past_fused(st.m, st.c2)) sums(std::false_type{});
+  else sums(std::true_type{});
   float p0, p1, w0, w1;
   unpack2(add2(s0, s1), p0, p1);
   st.s += p0 + p1;

@@ -148,3 +148,26 @@ def test_lm_head_pair_wait_runs_out():
     assert binding.read_device_status(ws) == (0, 0)
     ref = keep[0].double() @ keep[1].double().T
     assert torch.equal(out["row_argmax"].long().cpu(), ref.argmax(-1).cpu())
+
+
+@pytest.mark.parametrize("R", [40, 300])
+@pytest.mark.parametrize("T", [1.0, 0.1, 1e-2, 1e-3, 1e-6, 1e-8])
+def test_lm_head_sums_at_low_temperatures(R, T):
+    # Hidden states and weights are small integers, so every logit is exact and the sums are
+    # those of the row's differences: |max| / T reaches 3e10 where the weights' exponents are
+    # small. The exponents carry two roundings of at most 104 log2(e) 2^-23 for a weight above
+    # 2^-150: 1.8e-5 of it, and less than 1e-5 of a sum that holds the maximum's weight of 1.
+    rng = np.random.default_rng(R)
+    H, V = 64, 5003
+    h = rng.integers(-2, 3, (R, H)).astype(np.float32)
+    w = rng.integers(-8, 9, (V, H)).astype(np.float32)
+    w[rng.choice(V, 200, replace=False)] = w[0]  # ties
+    bits = lambda x: (x.view(np.uint32) >> 16).astype(np.uint16)  # exact in bf16
+    temp = np.full((R + 7) // 8, T, np.float32)
+    g = gpu_lm(bits(h), bits(w), temp, 8)
+    logits = h.astype(np.float64) @ w.T.astype(np.float64)
+    top = logits.max(1)
+    want = np.exp((logits - top[:, None]) / float(np.float32(T))).sum(1)
+    np.testing.assert_array_equal(g["row_max"], top)
+    np.testing.assert_array_equal(g["row_argmax"], logits.argmax(1))
+    np.testing.assert_allclose(g["row_sum"], want, rtol=1e-5)
