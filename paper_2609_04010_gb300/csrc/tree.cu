@@ -1020,9 +1020,9 @@ __global__ void __launch_bounds__(kThreads) tree_build_kernel(BuildParams p) {
   // pass 1, a 16-byte group at a time: the thread's maximum and its lowest index, the
   // sum of 2^((x - max) c2) (rescaled when the maximum rises), NaN or +inf seen (a NaN
   // sum, or a NaN among logits that are all -inf so far)
-  float m = -INFINITY, s = 0.f;
+  float m = -INFINITY, s = 0.f, mc = 0.f;
   int mi = -1;
-  bool nan_seen = false;
+  bool nan_seen = false, fused = false;  // fused: the exponents by one multiply-add (kFusedMax)
   for_groups<BF16, VEC>(rowp, e_begin, e_end, tid, [&](const auto& x, int base) {
     constexpr int E = sizeof(x) / sizeof(float);
     float vmax = x[0];
@@ -1036,12 +1036,16 @@ __global__ void __launch_bounds__(kThreads) tree_build_kernel(BuildParams p) {
       const int q0 = __ffs(eq) - 1;
       s *= ex2((m - vmax) * c2);
       m = vmax;
+      mc = m * c2;
+      fused = fabsf(mc) <= kFusedMax;
       mi = base + q0;
     }
-    if (m > -INFINITY) {
-      const float mc = m * c2;
+    if (fused) {
 #pragma unroll
       for (int q = 0; q < E; ++q) s += ex2(fmaf(x[q], c2, -mc));
+    } else if (m > -INFINITY) {
+#pragma unroll
+      for (int q = 0; q < E; ++q) s += ex2((x[q] - m) * c2);
     } else {
 #pragma unroll
       for (int q = 0; q < E; ++q) nan_seen |= x[q] != x[q];

@@ -505,3 +505,24 @@ def test_sampled_tree_bad_inputs_are_flagged():
         assert np.all(g["out_tokens"][b] == -1)
     for b in (0, 5):
         assert g["num_emitted"][b] == g["num_accepted"][b] + 2
+
+
+@pytest.mark.parametrize("V,dtype", [(4096, "bf16"), (4099, "bf16"), (4096, "f32"), (4099, "f32")])
+@pytest.mark.parametrize("shift", [20.0, -200.0])
+def test_build_tree_low_temperatures(oracle_mod, V, dtype, shift):
+    # |max| / T from 200 to 2e8: a row's log-sum is small where x / T and max / T are not. Two to
+    # five tokens share each row's maximum, so that the nodes' scores are sums of their counts'
+    # logarithms and the order of the nodes follows from them.
+    B, G, K, N = 8, 5, 6, 14
+    temps = np.resize(np.array([0.1, 1e-2, 1e-3, 1e-6], np.float32), B)
+    inp = W.make_accept_inputs(B, G, V, "f32", 3.0, 1.0, 1.0, seed=V)
+    rng = np.random.default_rng(V)
+    x = inp.drafter_logits.astype(np.float32) + np.float32(shift)
+    if dtype == "bf16":
+        x = torch.from_numpy(x).to(torch.bfloat16).float().numpy()
+    for b in range(B):
+        for j in range(G):
+            x[b, j, rng.choice(V, int(rng.integers(1, 5)), replace=False)] = x[b, j].max()
+    if dtype == "bf16":
+        x = (x.view(np.uint32) >> 16).astype(np.uint16)
+    check_build(oracle_mod, x, temps, inp.block_tokens[:, 0], K, N)
