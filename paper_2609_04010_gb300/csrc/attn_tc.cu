@@ -51,6 +51,7 @@ namespace specv {
 namespace {
 
 constexpr int TK = kTcKeyTile;               // keys per tile
+constexpr int kShortTiles = 3;               // units of at most as many tiles are never split
 
 // QR: query rows one Q or P buffer of an M tile holds: 128, or 64 when a KV group has at
 // most 64 query rows. The MMAs still read M = 128 rows; with QR = 64 the buffers are laid
@@ -572,7 +573,7 @@ __global__ void __launch_bounds__(TcCfg<D, MT, QR, HP>::THREADS, 1)
       // tree attention: the block keys this row sees (one bit per block position)
       const unsigned long long tmask =
           TREE ? __ldg(p.tree_mask + static_cast<int64_t>(s.b) * p.gamma + (ro.real ? ro.j : 0)) : 0ull;
-      float m = -INFINITY, l = 0.f;
+      float m = -INFINITY, l = 0.f, top = -INFINITY;  // top: the largest score (base 2) so far
       for (int k = 0; k < s.ntile; ++k) {
         const uint32_t x = it + k;
         ok = mbar_wait(s_full(mt, x & 1), (x >> 1) & 1, abort_flag, p.status);
@@ -622,8 +623,18 @@ __global__ void __launch_bounds__(TcCfg<D, MT, QR, HP>::THREADS, 1)
 #pragma unroll
           for (int c = 0; c < o; ++c) mx[c] = fmaxf(mx[c], mx[c + o]);
         const float tmax = mx[0] * p.scale_log2;  // base 2
-        const float m_new = fmaxf(m, tmax);
-        const bool want = k > 0 && m_new > m + (p.whole_units ? 0.f : 8.f);  // few tiles: the exact maximum
+        // The maximum that the probabilities are taken against is raised only past 2^8, except in
+        // short whole units: there each tile is taken against its own (or 2^-8 of the largest
+        // so far, so that nothing grows beyond that either), in which its largest probability
+        // is 1, exact in bf16, as in a part of a split unit: a relative error against 64 bits of
+        // 2.09e-3 at 64 to 256 rows over 128 to 500 keys, the same as in parts of one tile
+        // (2.11 to 2.15e-3 against the running maximum, 2.17 to 2.26e-3 past 2^8).
+        float m_new = fmaxf(m, tmax);
+        if (p.whole_units) {
+          top = fmaxf(top, tmax);
+          m_new = tmax > -INFINITY ? fmaxf(tmax, top - 8.f) : m;
+        }
+        const bool want = k > 0 && (p.whole_units ? m_new != m : m_new > m + 8.f);
         const bool rescale = __any_sync(0xffffffffu, want);
         float alpha = 1.f;
         if (k == 0) {
@@ -809,11 +820,21 @@ cudaError_t launch_typed(const spec_attn_args_t& a, const AttnPlan& P, char* ws,
   // keys and 256 rows 40.8 us in 152 ranges, 36.9 in 128.
   const int64_t k = P.grid / units, tiles = (p.max_keys + TK - 1) / TK;
   if (k > 0 && tiles * (P.grid - k * units) < 2 * Cf::UNIT_OVERHEAD * P.grid * k) p.grid = static_cast<int>(k * units);
-  // Short units that would be split in two at most are not split: 64 ragged units of up to
-  // 440 keys and 160 rows take 16.4 us whole, 28 split and merged. With fewer units, splitting
-  // them is as fast and more exact (each part's probabilities are rounded against its own
-  // maximum; 64 rows over 300 keys: a relative error of 2.09e-3 in parts, 2.16e-3 whole).
-  if (k <= 2 && tiles <= kWholeTiles) {
+  // Short units are not split: a dependent merge costs more than the tiles that splitting takes
+  // off a block, and a unit of one tile has nothing to split. Of up to three tiles, any number
+  // of units (us split and merged, now whole):
+  //   rows x units     1 tile        2 tiles       3 tiles
+  //    64 x 4       10.4  10.2    16.4  10.3    16.4  12.3
+  //    64 x 16      12.3  10.3    16.4  12.3    18.4  12.3
+  //   132 x 8       11.4  10.2    18.2  10.8    17.5  12.3
+  //   132 x 32      12.3  10.8    18.9  12.3    20.5  13.5
+  //   256 x 8       12.2  10.3    22.5  12.3    22.5  13.7
+  //   256 x 32      12.3  12.3    25.0  12.8    26.6  14.3
+  // Longer ones where a split would be in two at most: 64 ragged units of up to 440 keys and 160
+  // rows take 16.4 us whole, 28 split; but 4 units of 64 rows and 500 keys 14.4 split, and 64
+  // such units 20.5 whole. (The lengths are on the device: a page table that is wider than its
+  // contexts is split and merged, 4 units of 64 rows and one tile in 12.3 us.)
+  if (tiles <= kShortTiles || (k <= 2 && tiles <= kWholeTiles)) {
     p.grid = P.grid;
     p.whole_units = 1;
   }

@@ -268,3 +268,60 @@ def test_small_groups_bad_inputs_and_garbage(oracle_mod, gamma, head_dim, page):
         o_out, o_lse, st = oracle_attn(oracle_mod, inp)
         assert list(st) == [0, 1, 1, 0, 1]
         compare_attention(out.float().cpu().numpy(), lse.cpu().numpy(), o_out, o_lse)
+
+
+def check_whole_and_split(inp, tree_mask=None):
+    """A call whose page table is as wide as its contexts (short units whole in a block) against
+    the same call with a wide table (the general path: split by tiles and merged). Both take
+    each tile's probabilities against its own maximum, so they differ by fp32 rounding, which
+    may move a bf16 output to its neighbour (2^-7 of it), and in tiles 2^8 below a row's
+    maximum by their probabilities' rounding (2^-8 of a weight of 2^-8, on either side)."""
+    t = list(attn_tensors(inp))
+    out, lse = binding.verify_attention(*t, tree_mask=tree_mask)
+    pt = t[3]
+    t[3] = torch.full((pt.shape[0], 64), -1, dtype=pt.dtype, device=pt.device)
+    t[3][:, :pt.shape[1]] = pt
+    w_out, w_lse = binding.verify_attention(*t, tree_mask=tree_mask)
+    a, b = out.double(), w_out.double()
+    most = t[2].double().abs().max()
+    assert bool(((a - b).abs() <= 2.0 ** -7 * b.abs() + 2.0 ** -15 * most).all())
+    assert bool(((lse - w_lse).abs() <= 1e-5 + 2.0 ** -20 * w_lse.abs()).all())
+
+
+# Short units of the row-tile kernel (whole in a block whatever their number, up to three
+# 64-key tiles of the page table): one and two M tiles, head pairs, odd Hkv, a key on each
+# side of a tile's edge, and the first table that splits.
+@pytest.mark.parametrize("keys", [34, 64, 65, 128, 129, 192, 193])
+@pytest.mark.parametrize("batch,gamma,hq,hkv,dim", [(1, 33, 8, 8, 128), (2, 16, 8, 2, 128), (1, 33, 12, 3, 64),
+                                                    (3, 32, 8, 1, 128), (1, 32, 64, 2, 64), (2, 4, 3, 1, 128)])
+@pytest.mark.parametrize("tree", [False, True])
+def test_row_tile_short_units(batch, gamma, hq, hkv, dim, keys, tree):
+    inp = W.make_attn_inputs(batch, gamma, hq, hkv, dim, 16, keys - gamma, True, seed=keys + hq)
+    for b in range(1, batch):  # shorter ones in the same table
+        inp.kv_len[b] = max(gamma, keys - 41 * b)
+    masks = None
+    if tree:
+        rng = np.random.default_rng(keys)
+        masks = np.zeros((batch, gamma), np.uint64)
+        for b in range(batch):
+            for j in range(gamma):
+                up = masks[b, int(rng.integers(0, j))] if j else np.uint64(0)
+                masks[b, j] = up | np.uint64(1 << j)
+        masks = torch.from_numpy(masks.view(np.int64)).cuda()
+    check_whole_and_split(inp, masks)
+
+
+@pytest.mark.parametrize("gains", [(1.0, 12.0, 1.0), (12.0, 1.0, 1.0), (1.0, 1.0, 12.0), (12.0, 1.0, 12.0),
+                                   (0.01, 8.0, 0.5)])
+@pytest.mark.parametrize("gamma,hq,hkv", [(33, 8, 2), (32, 16, 2), (16, 8, 2)])
+def test_row_tile_short_units_falling_and_rising_maxima(gamma, hq, hkv, gains):
+    # three tiles of keys whose scores' scales differ by up to 16: each tile's probabilities are
+    # taken against its own maximum, more than 2^8 above or below the others'
+    inp = W.make_attn_inputs(2, gamma, hq, hkv, 128, 64, 192 - gamma, True, seed=77)
+    k = inp.k_cache
+    for b in range(2):
+        for t in range(3):
+            page = inp.page_table[b, t]
+            x = (k[page].astype(np.uint32) << 16).view(np.float32) * np.float32(gains[t])
+            k[page] = (torch.from_numpy(x).to(torch.bfloat16).view(torch.int16).numpy()).view(np.uint16)
+    check_whole_and_split(inp)
