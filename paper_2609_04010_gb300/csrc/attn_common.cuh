@@ -310,17 +310,28 @@ __device__ __forceinline__ void block_range(const AttnParams& p, const int* pb, 
     }
     return;
   }
-  const int per_b = p.hunits * p.row_tiles;
+  // Every role waits for this function, and a division is a chain of about 40 instructions: with
+  // a unit per block at most, two of them (six, as below: 64 units of one tile and 64 rows took
+  // 11.3 us instead of 10.3).
+  const uint32_t per_b = p.hunits * p.row_tiles;
   const int64_t units = static_cast<int64_t>(p.batch) * per_b;
+  if (units <= p.grid) {
+    if (cta < units) {
+      const uint32_t b = static_cast<uint32_t>(cta) / per_b;
+      const uint32_t len = static_cast<uint32_t>(pb[b + 1] - pb[b]) / per_b;
+      t0 = pb[b] + (static_cast<uint32_t>(cta) - b * per_b) * len;
+      t1 = t0 + len;
+    }
+    return;
+  }
   auto start = [&](int64_t u) -> int64_t {
     if (u >= units) return total;
     const int b = div_small(u, per_b);
-    return pb[b] + (static_cast<int>(u) - b * per_b) * ((pb[b + 1] - pb[b]) / per_b);
+    return pb[b] + (static_cast<int>(u) - b * static_cast<int>(per_b)) * ((pb[b + 1] - pb[b]) / static_cast<int>(per_b));
   };
-  const int64_t n = units < p.grid ? units : p.grid;
-  if (cta < n) {
-    t0 = start(div_small(cta * units, n));
-    t1 = start(div_small((cta + 1) * units, n));
+  if (cta < p.grid) {
+    t0 = start(div_small(cta * units, p.grid));
+    t1 = start(div_small((cta + 1) * units, p.grid));
   }
 }
 constexpr int kWholeTiles = 8;
