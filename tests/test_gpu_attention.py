@@ -325,3 +325,25 @@ def test_row_tile_short_units_falling_and_rising_maxima(gamma, hq, hkv, gains):
             x = (k[page].astype(np.uint32) << 16).view(np.float32) * np.float32(gains[t])
             k[page] = (torch.from_numpy(x).to(torch.bfloat16).view(torch.int16).numpy()).view(np.uint16)
     check_whole_and_split(inp)
+
+
+@pytest.mark.parametrize("gamma,hq,hkv,dim", [(1, 8, 2, 128), (4, 8, 2, 128), (8, 8, 2, 128), (4, 16, 4, 128),
+                                              (8, 16, 4, 128), (8, 16, 8, 64), (2, 12, 6, 64)])
+@pytest.mark.parametrize("keys,seed", [(120, 1), (128, 2), (113, 3), (33, 4)])
+def test_small_groups_short_units_falling_and_rising_maxima(oracle_mod, gamma, hq, hkv, dim, keys, seed):
+    # units of at most eight stages (one, two and four key groups) whose pages' scores differ in
+    # scale by up to 240, so that the stages' maxima rise and fall by far more than 2^2. P and
+    # the output are bf16 (2^-8 relative each): an element is off by at most 2^-7 of
+    # sum_k p_k |v_k| (the oracle's output with V's magnitudes), and 5% of it for the fp32 terms.
+    inp = W.make_attn_inputs(3, gamma, hq, hkv, dim, 16, keys - gamma, True, seed=seed)
+    gains = np.random.default_rng(seed).choice([0.05, 0.5, 1.0, 4.0, 12.0], inp.num_pages).astype(np.float32)
+    x = (inp.k_cache.astype(np.uint32) << 16).view(np.float32) * gains[:, None, None, None]
+    inp.k_cache[:] = torch.from_numpy(x).to(torch.bfloat16).view(torch.int16).numpy().view(np.uint16)
+    inp.kv_len[1] = max(gamma, keys - 37)
+    out, lse = gpu_attention(inp, binding.ATTN_AUTO)
+    args = (inp.page_table, inp.kv_len, gamma)
+    o_out, o_lse, st = oracle_mod.verify_attention(inp.q, inp.k_cache, inp.v_cache, *args)
+    o_abs, _, _ = oracle_mod.verify_attention(inp.q, inp.k_cache, inp.v_cache & np.uint16(0x7FFF), *args)
+    assert np.all(st == 0)
+    assert np.all(np.abs(out - o_out) <= 1.05 * 2.0 ** -7 * o_abs + 1e-6)
+    np.testing.assert_allclose(lse, o_lse, rtol=0, atol=1e-3)
