@@ -104,7 +104,7 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
 template <int D, int HB, int MTW>
 __global__ void __launch_bounds__(MmaCfg<D, HB, MTW>::THREADS, 1)
     attn_mma_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_constant__ CUtensorMap tmap_v,
-                    AttnParams p, int page_shift, int box_shift) {
+                    const __grid_constant__ AttnParams p, int page_shift, int box_shift) {
   using C = MmaCfg<D, HB, MTW>;
   constexpr int KS = C::KS, NS = C::NS, S = C::STAGES;
   const int box_keys = 1 << box_shift;  // keys per copy (page and box sizes are powers of two)
@@ -171,8 +171,7 @@ __global__ void __launch_bounds__(MmaCfg<D, HB, MTW>::THREADS, 1)
     for (Seg s = s_first; s.ntile > 0 && ok && !p.starve;) {
       for (int k = 0; k < s.ntile; ++k, ++it) {
         const uint32_t st = it % S;
-        if (it >= S) ok = mbar_wait_warp(empty(st), ((it / S) - 1) & 1, abort_flag, p.status);
-        if (!ok) break;
+        const bool free = it < S || mbar_wait(empty(st), ((it / S) - 1) & 1, abort_flag, p.status);
         const int key0 = (s.tile0 + k) * KS;
         // boxes with a visible key; a malformed sequence reads nothing
         const int nbox = s.len_ok ? min(KS >> box_shift, (s.kv_len - key0 + box_keys - 1) >> box_shift) : 0;
@@ -186,7 +185,7 @@ __global__ void __launch_bounds__(MmaCfg<D, HB, MTW>::THREADS, 1)
             bad |= !in_range;
             page[q] = in_range ? raw : 0;  // an out-of-range page is read as page 0
           }
-        if (lane == 0) {
+        if (lane == 0 && free) {
           if (warp == 0) stage_bad[st] = bad ? 1 : 0;
           if (nbox > 0) mbar_arrive_tx(full(st), nbox * box_bytes);
           else mbar_arrive(full(st));
@@ -196,7 +195,13 @@ __global__ void __launch_bounds__(MmaCfg<D, HB, MTW>::THREADS, 1)
               tma_load_group(ring + st * C::KV_BYTES + q * box_bytes, map, (key0 + (q << box_shift)) & (p.page_size - 1),
                              page[q] * p.hkv + s.g * HB, full(st));
         }
-        __syncwarp();
+        // a wait that ran out in some lanes ends the loop for all of them, after the shuffles
+        // of the page ids
+        ok = __all_sync(0xffffffffu, free);
+        if (!ok) {
+          it += __shfl_sync(0xffffffffu, free ? 1u : 0u, 0);  // whether this tile's copies were issued
+          break;
+        }
       }
       if (!ok || !has_more(s, t1, OVH)) break;
       s = locate<KS>(s.vnext, t1, p, pb, OVH);
@@ -516,9 +521,9 @@ __global__ void __launch_bounds__(MmaCfg<D, HB, MTW>::THREADS, 1)
       if (!has_more(s, t1, OVH)) break;
       s = locate<KS>(s.vnext, t1, p, pb, OVH);
     }
+    if (!ok && (lane & 3) == 0)
+      drop_partials<KS>(p, pb, r0 < p.rows ? h * p.rows + r0 : -1, r1 < p.rows ? h * p.rows + r1 : -1);
   }
-  __syncthreads();
-  if (*abort_flag) drop_partials<KS>(p, pb);
 }
 
 // ---------------------------------------------------------------------------------

@@ -159,7 +159,7 @@ template <int D, int MT, bool TREE, int QR, int HP>
 __global__ void __launch_bounds__(TcCfg<D, MT, QR, HP>::THREADS, 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
                    const __grid_constant__ CUtensorMap tmap_v,
-                   const __grid_constant__ CUtensorMap tmap_q, AttnParams p) {
+                   const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ AttnParams p) {
   using C = TcCfg<D, MT, QR, HP>;
   constexpr int SPLIT = C::SPLIT, KH = C::KH, PB = C::PB;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -786,10 +786,10 @@ __global__ void __launch_bounds__(TcCfg<D, MT, QR, HP>::THREADS, 1)
       s = sn;
       ++seg_no;
     }
+    if (!ok && hf == 0 && lrow < p.rows && lrow < p.rows_per_cta) drop_partials<TK>(p, pb, prow, -1);
     tc_fence_before();
   }
   __syncthreads();
-  if (*abort_flag) drop_partials<TK>(p, pb);
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, C::TMEM_COLS);
