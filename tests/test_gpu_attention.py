@@ -180,6 +180,8 @@ def test_deterministic_repeat():
 # The small-group kernel (automatic choice): 1 to 64 query rows per KV head (edges of its
 # 16-row tiles), 2, 4 and 8 KV heads per block, every page size, contexts that end inside
 # a 16-key step, units whole in a block, split over a few blocks and over many.
+# (The cases of 48, 49 and 64 rows are the row-tile kernel's: the small-group one takes up to
+# 32, whose edges are in test_rows_at_the_kernels_edges.)
 GROUPS = [
     dict(batch=1, gamma=1, num_q_heads=2, num_kv_heads=2, head_dim=128, page_size=16, ctx=0),
     dict(batch=24, gamma=1, num_q_heads=32, num_kv_heads=8, head_dim=128, page_size=16, ctx=(0, 900)),
@@ -347,3 +349,13 @@ def test_small_groups_short_units_falling_and_rising_maxima(oracle_mod, gamma, h
     assert np.all(st == 0)
     assert np.all(np.abs(out - o_out) <= 1.05 * 2.0 ** -7 * o_abs + 1e-6)
     np.testing.assert_allclose(lse, o_lse, rtol=0, atol=1e-3)
+
+
+@pytest.mark.parametrize("rows", [1, 15, 16, 17, 31, 32, 33, 34])  # up to 32: the small-group kernel
+@pytest.mark.parametrize("hkv,dim,page", [(4, 128, 16), (2, 128, 64), (8, 64, 32), (6, 64, 16)])
+def test_rows_at_the_kernels_edges(oracle_mod, rows, hkv, dim, page):
+    inp = W.make_attn_inputs(3, rows, hkv, hkv, dim, page, (100, 900), True, seed=300 + rows)
+    g_out, g_lse = gpu_attention(inp, binding.ATTN_AUTO)
+    o_out, o_lse, st = oracle_attn(oracle_mod, inp)
+    assert np.all(st == 0)
+    compare_attention(g_out, g_lse, o_out, o_lse)

@@ -234,3 +234,28 @@ def test_bound_beyond_the_near_values(oracle_mod):
     d = r["diag"].cpu().numpy()
     m = ~np.isnan(o["diag"])
     np.testing.assert_allclose(d[m], o["diag"][m], rtol=1e-4, atol=1e-9)
+
+
+@pytest.mark.parametrize("dtype,vocab", [("bf16", 4099), ("bf16", 33), ("bf16", 20001), ("f32", 4097), ("f32", 2049),
+                                         ("f32", 12290)])
+@pytest.mark.parametrize("shift", [0, 1, 3])
+@pytest.mark.parametrize("k,tp", [(20, 0.95), (200, 0.9)])
+def test_rows_at_every_alignment_against_the_oracle(oracle_mod, dtype, vocab, shift, k, tp):
+    # accepted lengths, tokens and probabilities of rows at every alignment, their tensors'
+    # neighbours NaN, excusing only sequences that the oracle marks as ties
+    B = 5
+    inp = W.make_accept_inputs(B, 4, vocab, dtype, 3.0, 0.5, [1.0, 0.0, 0.7], seed=300 + vocab + shift, draft_top_k=k)
+    t = list(accept_tensors(inp))
+    for i in (0, 1):
+        flat = torch.full((t[i].numel() + 16,), float("nan"), dtype=t[i].dtype, device="cuda")
+        flat[shift:shift + t[i].numel()] = t[i].flatten()
+        t[i] = flat[shift:shift + t[i].numel()].view(t[i].shape)
+    K, P = np.full(B, k, np.int32), np.full(B, tp, np.float32)
+    r = binding.accept_block_filtered(t[0], t[1], t[2], t[3], dev(K), dev(P), t[4])
+    torch.cuda.synchronize()
+    g = {key: v.cpu().numpy() for key, v in r.items() if v is not None}
+    o = oracle_filtered(oracle_mod, inp, K, P)
+    assert np.all(o["status"] == 0)
+    skip = {b for b in range(B) if o["filter_margin"][b] < FILTER_TIE and not same_outputs(g, o, b)}
+    compare_accept(g, o, inp.gamma, skip=skip)
+    assert len(skip) <= 1, skip
