@@ -40,6 +40,8 @@ struct AttnParams {
   int grid, min_tiles; // range_count: blocks launched, tiles a block takes at least
   int unit_heads;      // KV heads of a unit (attn_merge_kernel)
   int whole_units;     // ranges end at unit ends: nothing to merge (block_range)
+  float rise, fall;    // tensor cores: the running maximum (base 2) that probabilities are taken
+                       // against is raised past m + rise, and falls by at most `fall` a tile
   int starve;  // test hook: the producers issue no copies, so the consumers' waits run out
 };
 
@@ -83,6 +85,7 @@ inline AttnParams make_attn_params(const spec_attn_args_t& a, const AttnPlan& P,
   p.min_tiles = 1;
   p.unit_heads = 1;
   p.whole_units = 0;
+  p.rise = p.fall = 0.f;
   return p;
 }
 
@@ -351,14 +354,13 @@ __device__ __forceinline__ void note_split(const AttnParams& p, int cta, const S
   p.splits[cta] = d;
 }
 
-// A thread whose waits ran out leaves its rows (row0 and row1 of a slot, -1: none) without
-// their partials: in the slots of its block's first and last units (no other can be split) they
-// are marked bad, as a malformed sequence's are, so that those units' outputs become zeros
-// instead of what an earlier call left in the slots. A call, not inlined, and no barrier at the
-// block's end: with them a fused step of 8 requests of 8 positions took 48.3 us, now 47.6 (47.4
-// without any of this; the block's idle warps make room for the acceptance as they end).
+// A block whose waits ran out leaves units without their partials: rows first, first + step, ..
+// below end are marked bad in the slots of its first and last units (no other can be split), as
+// a malformed sequence's are, so that those units' outputs become zeros instead of what an
+// earlier call left in the slots. (The range is worked out again, so that the roles need not
+// keep it.)
 template <int TK>
-static __device__ __noinline__ void drop_partials(const AttnParams& p, const int* pb, int row0, int row1) {
+__device__ __forceinline__ void drop_partials(const AttnParams& p, const int* pb, int first, int end, int step) {
   const int64_t total = pb[p.batch];
   int64_t t0, t1;
   block_range(p, pb, blockIdx.x, total, range_count(total, p), t0, t1);
@@ -366,9 +368,17 @@ static __device__ __noinline__ void drop_partials(const AttnParams& p, const int
 #pragma unroll 1
   for (int i = 0; i < 2; ++i) {
     const int64_t slot = locate<TK>(i == 0 ? t0 : t1 - 1, t1, p, pb, p.unit_overhead).u + blockIdx.x;
-    if (row0 >= 0) p.partial_ml[slot * p.slot_rows + row0] = make_float2(-INFINITY, -1.f);
-    if (row1 >= 0) p.partial_ml[slot * p.slot_rows + row1] = make_float2(-INFINITY, -1.f);
+#pragma unroll 1
+    for (int r = first; r < end; r += step) p.partial_ml[slot * p.slot_rows + r] = make_float2(-INFINITY, -1.f);
   }
+}
+// The same as a call: a consumer thread of the small-group kernel marks its own rows. Inlined,
+// behind a barrier at the block's end, a fused step of 8 requests of 8 positions took 48.3 us,
+// with the call 47.6 (47.4 without any of this; the block's idle warps make room for the
+// acceptance as they end).
+template <int TK>
+static __device__ __noinline__ void drop_partials_call(const AttnParams& p, const int* pb, int first, int end, int step) {
+  drop_partials<TK>(p, pb, first, end, step);
 }
 
 // RW rows of one warp from their partial slots [slot0, slot0 + nsl), SB slots at a time: the

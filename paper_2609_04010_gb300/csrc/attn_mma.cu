@@ -339,8 +339,8 @@ __global__ void __launch_bounds__(MmaCfg<D, HB, MTW>::THREADS, 1)
         // and the times are within 0.7%.) In short whole units each stage is taken against its
         // own maximum, as a part of a split unit would be (falling by 2^2 a stage at most, 2^14
         // over a unit's eight, which the accumulators grow by): 2.03e-3 for 8 to 32 rows, two
-        // heads and up to 250 keys, as in parts, 2.05e-3 against the running maximum; 8 units
-        // of 32 rows take 13.3 us instead of 12.3. ----
+        // heads and up to 250 keys, as in parts, 2.05e-3 against the running maximum, in the same
+        // time (8 units of 32 rows 12.3 us). ----
         float x0 = -INFINITY, x1 = -INFINITY;
 #pragma unroll
         for (int n = 0; n < NS; ++n)
@@ -353,11 +353,7 @@ __global__ void __launch_bounds__(MmaCfg<D, HB, MTW>::THREADS, 1)
         x1 = fmaxf(x1, __shfl_xor_sync(0xffffffffu, x1, 1));
         x0 = fmaxf(x0, __shfl_xor_sync(0xffffffffu, x0, 2)) * p.scale_log2;
         x1 = fmaxf(x1, __shfl_xor_sync(0xffffffffu, x1, 2)) * p.scale_log2;
-        float n0 = fmaxf(m0, x0), n1 = fmaxf(m1, x1);
-        if (p.whole_units) {
-          n0 = x0 > -INFINITY ? fmaxf(x0, m0 - 2.f) : m0;
-          n1 = x1 > -INFINITY ? fmaxf(x1, m1 - 2.f) : m1;
-        }
+        const float n0 = fmaxf(x0, m0 - p.fall), n1 = fmaxf(x1, m1 - p.fall);
         if (__any_sync(0xffffffffu, n0 != m0 || n1 != m1)) {
           const float a0 = m0 == -INFINITY ? 0.f : ex2(m0 - n0), a1 = m1 == -INFINITY ? 0.f : ex2(m1 - n1);
           m0 = n0;
@@ -521,8 +517,8 @@ __global__ void __launch_bounds__(MmaCfg<D, HB, MTW>::THREADS, 1)
       if (!has_more(s, t1, OVH)) break;
       s = locate<KS>(s.vnext, t1, p, pb, OVH);
     }
-    if (!ok && (lane & 3) == 0)
-      drop_partials<KS>(p, pb, r0 < p.rows ? h * p.rows + r0 : -1, r1 < p.rows ? h * p.rows + r1 : -1);
+    if (!ok && (lane & 3) == 0)  // rows r0 and r1 = r0 + 8
+      drop_partials_call<KS>(p, pb, h * p.rows + r0, h * p.rows + min(p.rows, r1 + 1), 8);
   }
 }
 
@@ -571,6 +567,7 @@ cudaError_t launch_typed(const spec_attn_args_t& a, const AttnPlan& P, char* ws,
   p.unit_heads = HB;
   p.starve = starve ? 1 : 0;
   p.whole_units = p.max_keys <= kWholeTiles * C::KS ? 1 : 0;
+  p.fall = p.whole_units ? 2.f : 0.f;
   const size_t smem = C::smem_bytes(a.batch);
   auto kernel = attn_mma_kernel<D, HB, MTW>;
   const cudaError_t e = allow_smem(kernel, kTcMaxSmem);

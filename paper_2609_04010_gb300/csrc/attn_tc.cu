@@ -44,6 +44,8 @@
 // SPEC_FLAG_TIMEOUT, drains the block's own copies and MMAs, frees TMEM and exits.
 #include <cuda.h>  // CUtensorMap and its encoder's signature (resolved at run time)
 
+#include <algorithm>
+
 #include "attn_common.cuh"
 #include "tc_ptx.cuh"
 
@@ -159,7 +161,7 @@ template <int D, int MT, bool TREE, int QR, int HP>
 __global__ void __launch_bounds__(TcCfg<D, MT, QR, HP>::THREADS, 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap tmap_k,
                    const __grid_constant__ CUtensorMap tmap_v,
-                   const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ AttnParams p) {
+                   const __grid_constant__ CUtensorMap tmap_q, AttnParams p) {
   using C = TcCfg<D, MT, QR, HP>;
   constexpr int SPLIT = C::SPLIT, KH = C::KH, PB = C::PB;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -573,7 +575,7 @@ __global__ void __launch_bounds__(TcCfg<D, MT, QR, HP>::THREADS, 1)
       // tree attention: the block keys this row sees (one bit per block position)
       const unsigned long long tmask =
           TREE ? __ldg(p.tree_mask + static_cast<int64_t>(s.b) * p.gamma + (ro.real ? ro.j : 0)) : 0ull;
-      float m = -INFINITY, l = 0.f, top = -INFINITY;  // top: the largest score (base 2) so far
+      float m = -INFINITY, l = 0.f;
       for (int k = 0; k < s.ntile; ++k) {
         const uint32_t x = it + k;
         ok = mbar_wait(s_full(mt, x & 1), (x >> 1) & 1, abort_flag, p.status);
@@ -624,17 +626,14 @@ __global__ void __launch_bounds__(TcCfg<D, MT, QR, HP>::THREADS, 1)
           for (int c = 0; c < o; ++c) mx[c] = fmaxf(mx[c], mx[c + o]);
         const float tmax = mx[0] * p.scale_log2;  // base 2
         // The maximum that the probabilities are taken against is raised only past 2^8, except in
-        // short whole units: there each tile is taken against its own (or 2^-8 of the largest
-        // so far, so that nothing grows beyond that either), in which its largest probability
-        // is 1, exact in bf16, as in a part of a split unit: a relative error against 64 bits of
-        // 2.09e-3 at 64 to 256 rows over 128 to 500 keys, the same as in parts of one tile
-        // (2.11 to 2.15e-3 against the running maximum, 2.17 to 2.26e-3 past 2^8).
-        float m_new = fmaxf(m, tmax);
-        if (p.whole_units) {
-          top = fmaxf(top, tmax);
-          m_new = tmax > -INFINITY ? fmaxf(tmax, top - 8.f) : m;
-        }
-        const bool want = k > 0 && (p.whole_units ? m_new != m : m_new > m + 8.f);
+        // short whole units: there each tile is taken against its own (falling by 2^8 a tile at
+        // most, and 2^16 over a unit's tiles, which the accumulators grow by), in which its
+        // largest probability is 1, exact in bf16, as in a part of a split unit: a relative
+        // error against 64 bits of 2.09e-3 at 64 to 256 rows over 128 to 500 keys, the same as
+        // in parts of one tile (2.11 to 2.15e-3 against the running maximum, 2.17 to 2.26e-3
+        // past 2^8).
+        const float m_new = fmaxf(tmax, m - p.fall);
+        const bool want = k > 0 && (m_new > m + p.rise || m_new < m);
         const bool rescale = __any_sync(0xffffffffu, want);
         float alpha = 1.f;
         if (k == 0) {
@@ -786,10 +785,10 @@ __global__ void __launch_bounds__(TcCfg<D, MT, QR, HP>::THREADS, 1)
       s = sn;
       ++seg_no;
     }
-    if (!ok && hf == 0 && lrow < p.rows && lrow < p.rows_per_cta) drop_partials<TK>(p, pb, prow, -1);
     tc_fence_before();
   }
   __syncthreads();
+  if (*abort_flag) drop_partials<TK>(p, pb, threadIdx.x, p.slot_rows, C::THREADS);
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, C::TMEM_COLS);
@@ -838,6 +837,8 @@ cudaError_t launch_typed(const spec_attn_args_t& a, const AttnPlan& P, char* ws,
     p.grid = P.grid;
     p.whole_units = 1;
   }
+  p.rise = p.whole_units ? 0.f : 8.f;
+  p.fall = p.whole_units ? std::min(8.f, 16.f / std::max<int64_t>(tiles - 1, 1)) : 0.f;
   p.unit_heads = HP;
   if (!p.q_tma) mq = mk;  // unused
   const size_t smem = Cf::smem_bytes(a.batch);
