@@ -30,11 +30,11 @@ int device_sm_count(int dev) {
   return n;
 }
 
-// (Hq/Hkv) * gamma at and above which SPEC_ATTN_AUTO picks the tensor-core kernel.
-// Measured on GB300: the tensor-core kernel is never slower, from 4 rows per kv head
-// (equal time, both latency-bound) to 32 (6x faster: the CUDA-core kernel re-reads
-// each KV tile once per 16-row tile and issues the dot products on the FMA pipes), so
-// AUTO takes it whenever its shape limits allow.
+// (Hq/Hkv) * gamma at and above which SPEC_ATTN_AUTO picks a tensor-core kernel: always, where
+// the shape limits allow. The small-group kernel takes up to kMmaMaxRows rows per KV head (8
+// requests of 32 rows over 4,096 keys: 35 us), the row-tile kernel the rest; the CUDA-core
+// kernel re-reads each KV tile once per 16-row tile and issues the dot products on the FMA
+// pipes (300 us there).
 constexpr int kTcMinRows = 1;
 constexpr int kAcceptSms = 8;    // SMs a short attention leaves to a step's acceptance
 constexpr int kShortTiles = 64;  // 32 KB tiles per SM of a short attention

@@ -53,7 +53,7 @@ namespace specv {
 namespace {
 
 constexpr int TK = kTcKeyTile;               // keys per tile
-constexpr int kShortTiles = 3;               // units of at most as many tiles are never split
+constexpr int kUnsplitTiles = 3;               // units of at most as many tiles are never split
 
 // QR: query rows one Q or P buffer of an M tile holds: 128, or 64 when a KV group has at
 // most 64 query rows. The MMAs still read M = 128 rows; with QR = 64 the buffers are laid
@@ -833,7 +833,7 @@ cudaError_t launch_typed(const spec_attn_args_t& a, const AttnPlan& P, char* ws,
   // rows take 16.4 us whole, 28 split; but 4 units of 64 rows and 500 keys 14.4 split, and 64
   // such units 20.5 whole. (The lengths are on the device: a page table that is wider than its
   // contexts is split and merged, 4 units of 64 rows and one tile in 12.3 us.)
-  if (tiles <= kShortTiles || (k <= 2 && tiles <= kWholeTiles)) {
+  if (tiles <= kUnsplitTiles || (k <= 2 && tiles <= kWholeTiles)) {
     p.grid = P.grid;
     p.whole_units = 1;
   }
